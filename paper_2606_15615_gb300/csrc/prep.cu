@@ -230,9 +230,11 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(PrepArgs a) {
   // ---- A0: stage gate rows and token rows ----
   // Before the programmatic-dependency wait: everything that the previous
   // kernel (the layer below's combine) does not write.  The gate matrix is a
-  // weight; the cached metadata and the EMA rows were last written by this
-  // layer's own kernels one step earlier, which completed before the
-  // previous kernel could start.
+  // weight; the cached ids and weights and the EMA rows were last written by
+  // this kernel one step earlier, which completed before the previous kernel
+  // could start.  The cached norms come from the layer's combine, which is
+  // the previous kernel itself in a single-layer stack: they load after the
+  // wait.
   if (t == 0) {
     sm_near = 0;
     sm_nrows = 0;
@@ -263,7 +265,6 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(PrepArgs a) {
       for (int idx = t; idx < ntok * k; idx += kThreads) {
         sm_ce[idx] = a.sel.cache_e[cb + idx];
         sm_cw[idx] = a.sel.cache_w[cb + idx];
-        sm_cn[idx] = a.sel.cache_norm[cb + idx];
       }
     const size_t eb = static_cast<size_t>(tok0) * E;
     if (kRoute)
@@ -284,6 +285,8 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(PrepArgs a) {
     for (int q = lane; q < ntok; q += 32)
       bulk_g2s(smem_u32(s_x + q * ldw), x + static_cast<size_t>(tok0 + q) * D, row_bytes, bar);
   }
+  if (!a.sel.refresh)
+    for (int idx = t; idx < ntok * k; idx += kThreads) sm_cn[idx] = a.sel.cache_norm[static_cast<size_t>(tok0) * k + idx];
   if (!mbar_wait_for(bar, 0, kBarrierNs) && t == 0) report_status(a.status, kStatusWaitTimeout, 610);
   __syncthreads();
   // The grouped GEMM after this kernel reads the routed W1 first, expert by

@@ -320,3 +320,27 @@ def test_weight_prefetch_is_only_a_hint(M):
         for sa, sb in zip(states[0], states[other]):
             for key in ("cache_norm", "cache_h", "cache_e", "cache_w"):
                 assert torch.equal(sa[key], sb[key]), key
+
+
+def test_single_layer_steps_back_to_back(M):
+    """A one-layer stack: the layer's combine, which writes the cached norms,
+    is the kernel right before the next step's preparation kernel.  Steps
+    enqueued without a wait between them give the bits of steps with one."""
+    T, D, E, k, F = 512, 768, 16, 2, 3072
+    rng = np.random.default_rng(340)
+    xs = [torch.from_numpy(x).cuda().to(torch.bfloat16)
+          for x in drift(rng.standard_normal((T, D)).astype(np.float32), rng, 5, 0.05, True)]
+    outs = []
+    for wait in (True, False):
+        st, cfg, ws = make_stack(M, T, D, E, k, F, seed=34, tau0=0.64, wscale=0.02)
+        o = []
+        for t, x in enumerate(xs):
+            o.append(st.step(x, t))
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert 0 < st.stats()["reused"] < st.stats()["cache_step_branches"]
+        outs.append(o)
+        st.close()
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
