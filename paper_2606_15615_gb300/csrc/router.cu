@@ -126,6 +126,10 @@ __global__ void __launch_bounds__(NT) router_kernel(RouterArgs a, int stage_x, i
         sm_wg[(E + idx / rowv) * pstride + idx % rowv] = make_uint4(0, 0, 0, 0);
       for (int idx = t; idx < (TB - ntok) * rowv; idx += kThreads)
         sm_x[(ntok + idx / rowv) * pstride + idx % rowv] = make_uint4(0, 0, 0, 0);
+      // D an odd multiple of 8: the last 16-wide k-step takes in the rows' padding vector.
+      if (a.D % 16)
+        for (int r = t; r < epad + TB; r += kThreads)
+          (r < epad ? sm_wg + r * pstride : sm_x + (r - epad) * pstride)[rowv] = make_uint4(0, 0, 0, 0);
     }
     if (!mbar_wait_for(bar, 0, 1000000000ull) && t == 0) report_status(a.status, kStatusWaitTimeout, 500);
     if (tensor) __syncthreads();

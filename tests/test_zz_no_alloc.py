@@ -75,6 +75,12 @@ def test_noalloc_router_matches_moeca_step_twice(M, bf16):
     stack.close()
 
 
+@pytest.mark.parametrize("D,E,k", [(200, 16, 2), (328, 64, 4), (808, 8, 2), (1144, 64, 8)])
+def test_noalloc_router_width_an_odd_multiple_of_8(M, D, E, k):
+    """bf16 widths whose last 16-wide tensor-core step is half past the row."""
+    _noalloc_against_oracle(M, D, E, k, True)
+
+
 @pytest.mark.parametrize("D,bf16", [(1152, True), (1536, True), (1152, False)])
 def test_noalloc_wide_gate_router_against_oracle(M, D, bf16):
     """64 experts, top-8, 300 tokens (a ragged last block), two calls in a row,
@@ -83,7 +89,11 @@ def test_noalloc_wide_gate_router_against_oracle(M, D, bf16):
     router's wide-gate forms: 32-token blocks with the gate matrix and the
     token rows in shared memory together (D 1152, bf16), 16-token blocks with
     the token rows read through L1 (D 1536), and the fp32 form."""
-    T, E, k = 300, 64, 8
+    _noalloc_against_oracle(M, D, 64, 8, bf16)
+
+
+def _noalloc_against_oracle(M, D, E, k, bf16):
+    T = 300
     w, x0, rng = W.tiny_layer(41, T, D, E, k, 64, dtype="bf16" if bf16 else "f32", bias=True, wscale=0.05)
     cfg = M.moeca_config_default(n_layers=1, hidden=D, ffn=64, n_experts=E, top_k=k, max_tokens=T,
                                  dtype=M.MOECA_BF16 if bf16 else M.MOECA_F32, tau0=0.75)
