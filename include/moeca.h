@@ -87,9 +87,10 @@ typedef struct {
   int32_t reused_meta_policy; /* 0: a reused slot keeps w^{t0} (default); 1: it takes w^t */
   int32_t gelu_tanh;          /* 1: tanh-form GELU (default); 0: erf form */
   int32_t ffn_impl;           /* moeca_ffn_impl */
-  int32_t ffn_tile_n;         /* tensor-core FFN tile width: 0 = chosen per launch from the group
-                                 sizes (default), else 64 / 128 / 192 / 256 where it divides N */
-  int32_t ffn_split_k;        /* tensor-core FFN K splits: 0 = chosen per launch (default), else 1..4 */
+  int32_t ffn_tile_n;         /* widest token tile of the tensor-core FFN: 0 = 256 (default), else
+                                 64 / 128 / 192 / 256; each group's tiles are as narrow as its rows allow */
+  int32_t ffn_split_k;        /* K splits of the tensor-core FFN's second GEMM: 0 = none (default), else
+                                 1..4, where the launch's tiles fit the workspace */
   int32_t score_terms;        /* Eq. 9 terms in the branch score, a bit mask (Table 5's signal
                                  ablation): 1 = w, 2 = lambda1 Delta, 4 = lambda2 o; 7 (default) = all */
   int32_t granularity;        /* 0: branch-level decisions (MoECa, default); 1: token-level, a

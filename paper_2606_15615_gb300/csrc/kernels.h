@@ -104,8 +104,7 @@ struct FfnArgs {
   const int32_t* counts;
   const int32_t* offsets;
   const int32_t* list;
-  const void* xg;        // [rows, D]   gathered inputs (SIMT path)
-  const void* x;         // [T, D]      layer input: the tensor-core path gathers rows from it
+  const void* xg;        // [rows, D]   gathered inputs
   void* hmid;            // [rows, F]
   const void* w1;        // [E, F, D]
   const void* w2;        // [E, D, F]
@@ -114,13 +113,13 @@ struct FfnArgs {
   void* cache_h;         // [T*k, D]   destination rows of routed groups
   void* shared_h;        // [T, D]     destination rows of the shared group
   int gelu_tanh;
-  int tile_n;            // tensor-core tile width to force (0: chosen per launch)
+  int tile_n;            // tensor-core path: widest token tile to force (0: 256)
   int split_k;           // tensor-core K splits to force (0: chosen per launch)
   float* partial;        // split-K workspace: tensor-core path, or the fp32 path's [simt_split, max_rows, D]
   int simt_split;        // fp32 path: K splits of the second GEMM (1: none)
   int* tile_sem;         // split-K arrival counters, zeroed once
-  int* dep;              // tensor-core fused launch: per m-tile counter pairs, zeroed once (or null)
-  int max_mtiles;        // capacity of dep, tc_dep_pairs(max_rows, G)
+  int* dep;              // tensor-core path: per token-tile counter pairs, zeroed once
+  int dep_pairs;         // capacity of dep, tc_dep_pairs(max_rows, G)
   int* work;             // tensor-core path: unit ticket counter; 0 before every launch (the combine
                          // kernel that follows re-arms it)
   int* status;
@@ -131,13 +130,12 @@ cudaError_t launch_ffn_simt(const FfnArgs& a, bool bf16, int phase, cudaStream_t
 // handle; `TcPlan` owns them.
 struct TcPlan;
 TcPlan* tc_plan_create(const FfnArgs& a, int n_sms, char* err, int errlen);
-size_t tc_split_units(int n_sms);      // split-K units the workspace holds
+size_t tc_split_sems(int n_sms);       // split-K arrival counters of the workspace
 size_t tc_partial_bytes(int n_sms);    // bytes of the split-K partial workspace
-size_t tc_dep_pairs(int max_rows, int G);  // m-tile counter pairs a fused launch can need
+size_t tc_dep_pairs(int max_rows, int G);  // token-tile counter pairs a launch can need
 void tc_plan_destroy(TcPlan* p);
-// phase 1 or 2: that GEMM alone; phase 0: both, fused into one persistent
-// launch when a.dep is set and no K split is forced (else two launches).
-cudaError_t launch_ffn_tc(TcPlan* p, const FfnArgs& a, int phase, cudaStream_t s);
+// Both GEMMs in one persistent launch.
+cudaError_t launch_ffn_tc(TcPlan* p, const FfnArgs& a, cudaStream_t s);
 
 // Fused router + select + compact (one cooperative launch, bf16 only).
 struct PrepArgs {

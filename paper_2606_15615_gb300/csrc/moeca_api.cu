@@ -66,13 +66,6 @@ namespace {
 
 thread_local std::string g_create_error;
 
-// Phase 1 of the tensor-core FFN can gather its A rows from the layer input
-// with TMA tile::gather4 instead of reading rows that compact_kernel copied
-// into a contiguous buffer.  Measured on GB300 the gather issue rate (32
-// gather4 per 64-wide k-block from one thread) costs more than the copy, so
-// the copy path is the default.
-constexpr bool kGemmGathersRows = false;
-
 struct LayerBuf {
   moeca_layer_weights w;
   int32_t* cache_e = nullptr;
@@ -127,7 +120,7 @@ struct moeca_handle {
   float* simt_partial = nullptr;  // fp32 path: second-GEMM K-split partials [simt_split, max_rows, D]
   int simt_split = 1;
   int* tc_sem = nullptr;
-  int* tc_dep = nullptr;        // fused GEMM launch: m-tile dependency counters, left at 0
+  int* tc_dep = nullptr;        // grouped GEMM: token-tile dependency counters, left at 0
   int* tc_work = nullptr;       // GEMM unit tickets {next, CTAs done}, left at 0
   int tc_dep_pairs_n = 0;
   PrepShape prep{0, 0, 0, 0, false};  // fused router + select + compact, when it fits
@@ -326,18 +319,18 @@ PrepArgs prep_args_plain(const moeca_handle* h, const LayerBuf& L, const void* m
   return pa;
 }
 
-FfnArgs ffn_args(const moeca_handle* h, const LayerBuf& L, int T, const void* moe_in) {
+FfnArgs ffn_args(const moeca_handle* h, const LayerBuf& L, int T) {
   const moeca_config& c = h->cfg;
   FfnArgs fa{};
   fa.G = h->G; fa.E = c.n_experts; fa.D = c.hidden; fa.F = c.ffn; fa.k = c.top_k; fa.T = T;
   fa.max_rows = T * (c.top_k + c.n_shared);
   fa.counts = L.counts; fa.offsets = L.offsets; fa.list = L.list;
-  fa.xg = h->xg; fa.hmid = h->hmid; fa.x = kGemmGathersRows ? moe_in : nullptr;
+  fa.xg = h->xg; fa.hmid = h->hmid;
   fa.w1 = L.w.w1; fa.w2 = L.w.w2; fa.ws1 = L.w.ws1; fa.ws2 = L.w.ws2;
   fa.cache_h = L.cache_h; fa.shared_h = L.shared_h; fa.gelu_tanh = c.gelu_tanh; fa.status = h->status_dev;
   fa.partial = h->simt_partial ? h->simt_partial : h->tc_partial; fa.tile_sem = h->tc_sem;
   fa.simt_split = h->simt_split;
-  fa.dep = h->tc_dep; fa.max_mtiles = h->tc_dep_pairs_n; fa.work = h->tc_work;
+  fa.dep = h->tc_dep; fa.dep_pairs = h->tc_dep_pairs_n; fa.work = h->tc_work;
   return fa;
 }
 
@@ -582,7 +575,7 @@ moeca_status moeca_create(const moeca_config* cfg, const moeca_layer_weights* la
   }
   if (use_tc) {
     A((void**)&h->tc_partial, tc_partial_bytes(h->n_sms));
-    A((void**)&h->tc_sem, tc_split_units(h->n_sms) * sizeof(int));
+    A((void**)&h->tc_sem, tc_split_sems(h->n_sms) * sizeof(int));
     h->tc_dep_pairs_n = static_cast<int>(tc_dep_pairs(h->max_rows, h->G));
     A((void**)&h->tc_dep, static_cast<size_t>(h->tc_dep_pairs_n) * 2 * sizeof(int));
     A((void**)&h->tc_work, 2 * sizeof(int));
@@ -619,7 +612,7 @@ moeca_status moeca_create(const moeca_config* cfg, const moeca_layer_weights* la
       fa.max_rows = h->max_rows;
       fa.xg = h->xg; fa.hmid = h->hmid;
       fa.w1 = L.w.w1; fa.w2 = L.w.w2; fa.ws1 = L.w.ws1; fa.ws2 = L.w.ws2;
-      fa.tile_n = c.ffn_tile_n; fa.split_k = c.ffn_split_k;
+      fa.tile_n = c.ffn_tile_n; fa.split_k = c.ffn_split_k; fa.gelu_tanh = c.gelu_tanh;
       char err[256] = {0};
       L.tc = tc_plan_create(fa, h->n_sms, err, sizeof err);
       if (!L.tc) {
@@ -774,8 +767,7 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
     }
     // Under the sync rule the rows' inputs change after the decision: the
     // FFN rows are gathered once the attention update is done.
-    const bool xg_gather = !(use_tc && kGemmGathersRows);  // the FFN reads gathered rows
-    void* xg_now = !xg_gather || attn_sync ? nullptr : h->xg;
+    void* xg_now = attn_sync ? nullptr : h->xg;
 
     const bool fused = h->prep.tokens_per_block != 0;
     RouterArgs ra{};
@@ -808,7 +800,7 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
         pa.attn_rows = h->attn_rows; pa.attn_n = h->attn_n; pa.attn_inv = h->attn_inv;
         pa.sample_lo = h->attn_samp; pa.seq = seq;
       }
-      if (attn_sync && !ada && xg_gather) {
+      if (attn_sync && !ada) {
         // The rows of tokens that keep their attention are final now; the
         // output projection writes the others (row_of says where).
         pa.xg = h->xg;
@@ -847,7 +839,7 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
         mm.m_out = L.attn_m; mm.rows = h->attn_rows; mm.n_rows = h->attn_n;
         if ((e = timed(h, MOECA_K_ADALN, s, [&] { return launch_adaln_rows(mm, s); })) != cudaSuccess) break;
       }
-      if (xg_gather && (!fused || ada)) {
+      if (!fused || ada) {
         CompactArgs ga = ca;
         ga.xg = h->xg;
         if ((e = timed(h, MOECA_K_ATTN_AUX, s, [&] { return launch_gather(ga, h->bf16, s); })) != cudaSuccess)
@@ -855,17 +847,15 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
       }
     }
 
-    FfnArgs fa = ffn_args(h, L, T, moe_in);
+    FfnArgs fa = ffn_args(h, L, T);
     if (use_tc) {
       // Both GEMMs in one persistent launch: phase-2 tiles start as soon as
       // the phase-1 tiles of their rows are stored.
-      e = timed(h, MOECA_K_FFN, s, [&] { return launch_ffn_tc(L.tc, fa, 0, s); });
+      e = timed(h, MOECA_K_FFN, s, [&] { return launch_ffn_tc(L.tc, fa, s); });
     } else {
       for (int phase = 1; phase <= 2 && e == cudaSuccess; ++phase) {
         const int kind = phase == 1 ? MOECA_K_FFN1 : MOECA_K_FFN2;
-        e = timed(h, kind, s, [&] {
-          return use_tc ? launch_ffn_tc(L.tc, fa, phase, s) : launch_ffn_simt(fa, h->bf16, phase, s);
-        });
+        e = timed(h, kind, s, [&] { return launch_ffn_simt(fa, h->bf16, phase, s); });
       }
     }
     if (e != cudaSuccess) break;
@@ -992,8 +982,8 @@ cudaError_t shard_finish(moeca_handle* h, int l, const void* in, void* out, cuda
   pa.epoch = pa.wait_epoch = h->prep_epoch;
   cudaError_t e = timed(h, MOECA_K_PREP, s, [&] { return launch_prep_shard(pa, h->prep, 2, s); });
   if (e != cudaSuccess) return e;
-  FfnArgs fa = ffn_args(h, L, T, in);
-  if ((e = timed(h, MOECA_K_FFN, s, [&] { return launch_ffn_tc(L.tc, fa, 0, s); })) != cudaSuccess) return e;
+  FfnArgs fa = ffn_args(h, L, T);
+  if ((e = timed(h, MOECA_K_FFN, s, [&] { return launch_ffn_tc(L.tc, fa, s); })) != cudaSuccess) return e;
   const CombineArgs cb = combine_args(h, L, T, in, out, h->sh.refresh, true);
   return timed(h, MOECA_K_COMBINE, s, [&] { return launch_combine(cb, h->bf16, s); });
 }
@@ -1246,7 +1236,7 @@ moeca_status moeca_reset(moeca_handle* h) {
   // Counters that kernels leave at zero, unless a launch was cut short.
   if (h->tc_dep) {
     cudaError_t e = cudaMemset(h->tc_dep, 0, static_cast<size_t>(h->tc_dep_pairs_n) * 2 * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(h->tc_sem, 0, tc_split_units(h->n_sms) * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(h->tc_sem, 0, tc_split_sems(h->n_sms) * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->tc_work, 0, 2 * sizeof(int));
     if (e != cudaSuccess) return cuda_fail(h, e, "reset GEMM counters");
   }
