@@ -229,18 +229,15 @@ cudaError_t launch_combine(const CombineArgs& a, bool bf16, cudaStream_t s);
 // ---- Attention path of a DiT-MoE block (Sec. 4.1), bf16 only ----
 
 // Tensor-core projection GEMM: C = A B^T + bias (proj_tc.cu).
-enum ProjMode { kProjStore = 0, kProjResidual = 1, kProjQKV = 2, kProjResidualGated = 3 };
+enum ProjMode { kProjResidual = 1, kProjQKV = 2, kProjResidualGated = 3 };
 struct ProjArgs {
   const void* A;          // [a_rows, K] bf16, row-major
   int a_rows;             // rows A holds (>= M)
   const void* B;          // [N, K] bf16 weights
   const float* bias;      // [N] or null
   int M, N, K;            // N a multiple of 64, K of 64
-  int tile_n;             // output tile width (0: the widest of 256 / 128 / 64 dividing N)
   const int* m_dev;       // device row count (<= M), or null
   int mode;               // ProjMode
-  void* out;              // kProjStore: [M, ldo] bf16
-  int ldo;
   const int32_t* rows;    // kProjResidual: token of row m, or null (m)
   int n_tok;              // kProjResidual: rows of x / a_out / u_out
   const void* x;          // kProjResidual: [n_tok, N]
@@ -258,10 +255,7 @@ struct ProjArgs {
   int gate_ld, seq;       //   gate + (t / seq) * gate_ld (AdaLN block)
   int* status;
 };
-// Tile width a launch uses for N: `want` (64 / 128 / 256) if it divides N,
-// else (want = 0) the widest that does; 0 when none fits.
-int proj_tile_n(int N, int want);
-cudaError_t launch_proj_tc(const ProjArgs& a, cudaStream_t s);
+cudaError_t launch_proj_tc(const ProjArgs& a, int n_sms, cudaStream_t s);
 
 // ---- AdaLN modulation of a DiT-MoE block (Sec. 3) and the sampler step (Eq. 1) ----
 

@@ -715,12 +715,6 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
     ProjArgs oa{};
     oa.A = h->attn_o; oa.a_rows = T; oa.B = L.w.w_o; oa.bias = L.w.b_o;
     oa.M = T; oa.N = c.hidden; oa.K = c.hidden; oa.mode = kProjResidual;
-    // Narrow tiles at moderate width: the recomputed rows are few and the
-    // residual epilogue (x in; a, u and the FFN rows out) is latency-bound,
-    // so more CTAs with two 32-column chunks each beat fewer wide ones.  At
-    // D above 2048 the K loop dominates and narrow tiles would re-read the
-    // operands four times over: the widest tile.
-    oa.tile_n = c.hidden > 2048 ? 0 : 64;
     oa.n_tok = T; oa.x = in; oa.a_out = L.attn_a; oa.u_out = L.attn_u;
     if (ada) {
       oa.mode = kProjResidualGated;
@@ -739,11 +733,11 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
         ha.h_out = h->ada_h;
         if ((e = timed(h, MOECA_K_ADALN, s, [&] { return launch_adaln_rows(ha, s); })) != cudaSuccess) break;
       }
-      if ((e = timed(h, MOECA_K_QKV, s, [&] { return launch_proj_tc(qa, s); })) != cudaSuccess) break;
+      if ((e = timed(h, MOECA_K_QKV, s, [&] { return launch_proj_tc(qa, h->n_sms, s); })) != cudaSuccess) break;
       if ((e = timed(h, MOECA_K_ATTN, s, [&] {
              return use_attn_tc ? launch_attn_tc(aa, s) : launch_attn_core(aa, s);
            })) != cudaSuccess) break;
-      if ((e = timed(h, MOECA_K_OPROJ, s, [&] { return launch_proj_tc(oa, s); })) != cudaSuccess) break;
+      if ((e = timed(h, MOECA_K_OPROJ, s, [&] { return launch_proj_tc(oa, h->n_sms, s); })) != cudaSuccess) break;
       if (ada) {
         AdaLnArgs mm = la;
         mm.m_out = L.attn_m; mm.m_copy = L.route_m;
@@ -828,11 +822,11 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
                                                h->attn_inv, s);
                      })) != cudaSuccess)
         break;
-      if ((e = timed(h, MOECA_K_QKV, s, [&] { return launch_proj_tc(qa, s); })) != cudaSuccess) break;
+      if ((e = timed(h, MOECA_K_QKV, s, [&] { return launch_proj_tc(qa, h->n_sms, s); })) != cudaSuccess) break;
       if ((e = timed(h, MOECA_K_ATTN, s, [&] {
              return use_attn_tc ? launch_attn_tc(aa, s) : launch_attn_core(aa, s);
            })) != cudaSuccess) break;
-      if ((e = timed(h, MOECA_K_OPROJ, s, [&] { return launch_proj_tc(oa, s); })) != cudaSuccess) break;
+      if ((e = timed(h, MOECA_K_OPROJ, s, [&] { return launch_proj_tc(oa, h->n_sms, s); })) != cudaSuccess) break;
       if (ada) {
         // The listed tokens' MoE input m from their new u.
         AdaLnArgs mm = la;

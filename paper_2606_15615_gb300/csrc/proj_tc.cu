@@ -5,8 +5,7 @@
 //
 // with A [rows, K] row-major (the block input for the query / key / value
 // projection, the attention rows for the output projection) and B [N, K] a
-// weight matrix.  Two epilogues:
-//   kProjStore     out[m, n] = bf16(C[m, n])
+// weight matrix.  Epilogues:
 //   kProjQKV       N = 3D split into the attention's operand layouts: the q
 //                  columns of token m go to row inv[m] of q_out (the token's
 //                  place in the recomputing-token list; none if -1), the k
@@ -19,26 +18,33 @@
 //   kProjResidualGated  as kProjResidual with u = bf16(x + g a), g the row's
 //                  AdaLN gate (the sample's gate vector, Sec. 3); no FFN rows
 // M is a host bound; when m_dev is set the launch reads the actual row count
-// there (rows recomputed this step) and tiles past it return at once.
+// there (rows recomputed this step).
 //
-// One CTA per 128 x BN output tile, 6 warps:
-//   warp 0    TMA producer: A 128 x 64 and B BN x 64 per stage, 128-byte
-//             swizzle, into a ring of `nst` stages;
-//   warp 1    allocates BN TMEM columns and issues tcgen05.mma (M = 128,
-//             N = BN, K = 16) from one thread; tcgen05.commit frees a stage
-//             and finally signals the finished accumulator;
-//   warps 2-5 epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (its rows),
-//             32 columns at a time, and adds the bias (staged in shared memory
-//             while the MMAs run).  Store mode rounds to bf16 and writes
-//             through a 2 KB shared-memory stage, so each store covers 64
-//             contiguous bytes of 8 rows; residual mode loads the token's x
-//             one chunk ahead and writes a and u, 64 bytes per lane.
+// Persistent CTA pairs (clusters of two, cta_group::2) as in the grouped FFN:
+// a tile is 256 weight rows (the MMA's M side, 128 per CTA) by `n` token rows
+// (its N side, half per CTA), two K sub-blocks of 64 per stage.  Tiles go to
+// the pairs round robin, token tile by token tile.  11 warps per CTA:
+//   warp 0    TMA producer of the weight boxes (128 rows);
+//   warp 10   TMA producer of the token boxes (n / 2 rows);
+//   warp 1    allocates 512 TMEM columns; in the leader, one thread issues
+//             tcgen05.mma (M = 256, N = n, K = 16) for both CTAs into one of two
+//             accumulators, so a tile's epilogue overlaps the next tile's MMAs;
+//   warps 2-9 epilogue of the CTA's 128 features (TMEM lanes), two warps per
+//             lane quadrant, each half of the token columns: 32 features x 32
+//             tokens at a time through a 2 KB shared-memory stage, transposed
+//             (except v^T, which wants the features' rows), so that each
+//             global access covers 64 contiguous bytes of 8 rows.
+// A kernel of single CTAs with one 128 x BN tile each was bound by its operand
+// fill and by the CTAs' start and end.  Event-timed per launch on GB300, that
+// one -> this one (4096 rows, cache steps with 60% of the rows listed):
+//   D 1152 q/k/v 74 -> 32, 69 -> 28 us; output projection 49 -> 23, 42 -> 24 us
+//   D 768 (2048 rows) q/k/v 19 -> 20, 16 -> 16 us; output 22 -> 14, 16 -> 15 us
 // Every wait is bounded (about one second); a wait that runs out records the
 // timeout status, raises a CTA abort flag, waits (bounded) for the copies and
 // MMAs already issued, frees TMEM and returns.
 #include <cuda.h>
 
-#include <cstdio>
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -49,24 +55,30 @@ namespace moeca {
 
 namespace {
 
-constexpr int kPM = 128;
-constexpr int kPThreads = 192;
-constexpr int kPABytes = kPM * 64 * 2;  // 16 KB: A box of one stage
-constexpr int kPEpiStage = 32 * 64;     // per epilogue warp: 32 rows x 32 bf16
+constexpr int kBM = 128;                // weight rows per CTA (half of the MMA's M)
+constexpr int kBK = 64;                 // K per sub-block
+constexpr int kSub = 2;                 // K sub-blocks per stage
+constexpr int kMaxN = 256;              // token rows per tile
+constexpr int kBoxes = kMaxN / 32;      // token boxes of 16, 32, .., 128 rows
+constexpr int kMaxStages = 5;
+constexpr int kRingBytes = 208 * 1024;
+constexpr int kABytes = kBM * kBK * 2;  // 16 KB: one weight sub-block
+constexpr int kEpiWarps = 8;            // warps 2-9
+constexpr int kTokWarp = 2 + kEpiWarps;
+constexpr int kPThreads = 32 * (kTokWarp + 1);
+constexpr int kStageOut = 32 * 64;      // per epilogue warp: 32 x 32 bf16
+constexpr int kPSmem = kRingBytes + kEpiWarps * kStageOut + 1024;
+constexpr int kTmemCols = 512;
 
 struct ProjParams {
   int M, N, K;
   const int* m_dev;          // device row count (<= M), or null: M rows
   const float* bias;         // [N] or null
-  int mode;                  // ProjMode
-  __nv_bfloat16* out;        // kProjStore: [M, ldo]
-  int ldo;
   const int32_t* rows;       // kProjResidual: token of row m, or null (m)
   int n_tok;                 // kProjResidual: tokens the x / a_out / u_out rows hold
   const __nv_bfloat16* x;    // kProjResidual: [n_tok, N]
   __nv_bfloat16* a_out;      // kProjResidual: [n_tok, N]
   __nv_bfloat16* u_out;      // kProjResidual: [n_tok, N]
-  int nst;                   // ring stages
   unsigned long long* row_stat;
   const int32_t* row_of;     // kProjResidual: [n_tok, row_w] FFN rows of the token (-1: none), or null
   int row_w;
@@ -80,368 +92,376 @@ struct ProjParams {
   int* status;
 };
 
-constexpr int kMaxRowOf = kMaxTopK + 1;
+struct ProjMaps {
+  CUtensorMap w;             // weights, box 128 rows
+  CUtensorMap act[kBoxes];   // token rows, boxes of 16 .. 128 rows
+};
 
-// Store mode, one warp's 32 x 32 chunk: lane i holds row i's 32 values
-// (bias added).  They are rounded to bf16 and staged, then written 16 bytes
-// per lane with four lanes per row, so each store covers 64 contiguous bytes
-// of 8 rows.  `dst` is this lane's row at the chunk's first column (null:
-// not stored).
-__device__ __forceinline__ void store_chunk_staged(uint8_t* stage, const float* v, __nv_bfloat16* dst, int lane) {
-  uint32_t packed[16];
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    __nv_bfloat162 h2 = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-    packed[j] = *reinterpret_cast<uint32_t*>(&h2);
+// Token tile width for `rows` rows: the fewest waves x time per tile.  A
+// tile's time per stage is its MMAs' (an M 256 MMA takes as long at N 128 as at
+// 256) plus a share that grows with the token rows brought in.
+__device__ __forceinline__ int token_width(int rows, int nw, int pairs) {
+  int best = 256, best_cost = 0x7fffffff;
+  for (int n = 256; n >= 32; n -= 32) {
+    const int tiles = (rows + n - 1) / n * nw;
+    const int cost = (tiles + pairs - 1) / pairs * (384 + n);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = n;
+    }
   }
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    *reinterpret_cast<uint4*>(stage + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) =
-        make_uint4(packed[4 * j], packed[4 * j + 1], packed[4 * j + 2], packed[4 * j + 3]);
-  __syncwarp();
-  const unsigned long long d_mine = reinterpret_cast<unsigned long long>(dst);
-#pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    const int row = it * 8 + (lane >> 2), j = lane & 3;
-    const uint4 val = *reinterpret_cast<const uint4*>(stage + row * 64 + ((j ^ ((row >> 1) & 3)) << 4));
-    __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(__shfl_sync(0xffffffffu, d_mine, row));
-    if (d) *reinterpret_cast<uint4*>(d + j * 8) = val;
-  }
-  __syncwarp();
+  return best;
 }
 
-// q/k/v mode, v columns: the warp's 32 x 32 chunk transposed through the
-// stage, so each lane writes 16 bytes (8 consecutive tokens) of one v^T row.
-// `vt` is v^T's row of the chunk's first column, `tok0` the warp's first
-// token (a multiple of 32), `M` the token count (a multiple of 8).
-__device__ __forceinline__ void store_chunk_transposed(uint8_t* stage, const float* v, __nv_bfloat16* vt, int tok0,
-                                                       int M, size_t ld, int lane) {
-  __nv_bfloat16* st = reinterpret_cast<__nv_bfloat16*>(stage);  // [32 columns][32 tokens]
-#pragma unroll
-  for (int j = 0; j < 32; ++j) st[j * 32 + lane] = __float2bfloat16_rn(v[j]);
-  __syncwarp();
-#pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    const int j = it * 8 + (lane >> 2), seg = lane & 3;
-    const int tok = tok0 + seg * 8;
-    if (tok < M)
-      *reinterpret_cast<uint4*>(vt + static_cast<size_t>(j) * ld + tok) =
-          *reinterpret_cast<const uint4*>(st + j * 32 + seg * 8);
-  }
-  __syncwarp();
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<uint32_t*>(&h2);
 }
 
-// Residual mode, one lane's row: a = bf16(v), u = bf16(x + a), each 64
-// contiguous bytes (two full 32-byte sectors) written by the lane itself;
-// u also goes to the token's FFN input rows (g_dst[q], or null).
-__device__ __forceinline__ void store_residual(const float* v, const uint4* xv, __nv_bfloat16* a_dst,
-                                               __nv_bfloat16* u_dst, __nv_bfloat16* const* g_dst, int n_g) {
+// A warp's 32 features (lanes) x 32 tokens as bf16 into the stage
+// [32 tokens][32 features]: lanes 2i and 2i + 1 swap halves, so that each holds
+// the feature pair of every other token and the 32 words of a store fall in
+// 32 banks.
+__device__ __forceinline__ void stage_by_token(uint32_t* stage, const uint32_t* v, float bias, int lane) {
+  const uint32_t odd = lane & 1;
+#pragma unroll
+  for (int t = 0; t < 16; ++t) {
+    const uint32_t own = pack_bf16(__uint_as_float(v[2 * t]) + bias, __uint_as_float(v[2 * t + 1]) + bias);
+    const uint32_t got = __shfl_xor_sync(0xffffffffu, own, 1);
+    stage[(2 * t + odd) * 16 + (lane >> 1)] = odd ? __byte_perm(got, own, 0x7632) : __byte_perm(own, got, 0x5410);
+  }
+}
+
+// The same as [32 features][32 tokens], 16-byte chunks XOR-swizzled by row
+// pairs so that both accesses are conflict-free.
+__device__ __forceinline__ void stage_by_feature(uint32_t* stage, const uint32_t* v, float bias, int lane) {
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    uint4 av, uv;
-    __nv_bfloat162* ah = reinterpret_cast<__nv_bfloat162*>(&av);
-    __nv_bfloat162* uh = reinterpret_cast<__nv_bfloat162*>(&uv);
-    const __nv_bfloat162* xh = reinterpret_cast<const __nv_bfloat162*>(&xv[j]);
+    uint4 w;
+    uint32_t* wp = reinterpret_cast<uint32_t*>(&w);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      ah[q] = __floats2bfloat162_rn(v[8 * j + 2 * q], v[8 * j + 2 * q + 1]);
-      const float2 af = __bfloat1622float2(ah[q]);
-      const float2 xf = __bfloat1622float2(xh[q]);
-      uh[q] = __floats2bfloat162_rn(xf.x + af.x, xf.y + af.y);
-    }
-    reinterpret_cast<uint4*>(a_dst)[j] = av;
-    reinterpret_cast<uint4*>(u_dst)[j] = uv;
-#pragma unroll
-    for (int q = 0; q < kMaxRowOf; ++q)
-      if (q < n_g && g_dst[q]) reinterpret_cast<uint4*>(g_dst[q])[j] = uv;
+    for (int q = 0; q < 4; ++q)
+      wp[q] = pack_bf16(__uint_as_float(v[8 * j + 2 * q]) + bias, __uint_as_float(v[8 * j + 2 * q + 1]) + bias);
+    reinterpret_cast<uint4*>(stage)[lane * 4 + (j ^ ((lane >> 1) & 3))] = w;
   }
 }
 
-// Gated residual (AdaLN block): a = bf16(v), u = bf16(x + g a), 32 columns.
-__device__ __forceinline__ void store_residual_gated(const float* v, const uint4* xv, const float* g,
-                                                     __nv_bfloat16* a_dst, __nv_bfloat16* u_dst) {
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float4 g0 = __ldg(reinterpret_cast<const float4*>(g + 8 * j));
-    const float4 g1 = __ldg(reinterpret_cast<const float4*>(g + 8 * j) + 1);
-    const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-    uint4 av, uv;
-    __nv_bfloat162* ah = reinterpret_cast<__nv_bfloat162*>(&av);
-    __nv_bfloat162* uh = reinterpret_cast<__nv_bfloat162*>(&uv);
-    const __nv_bfloat162* xh = reinterpret_cast<const __nv_bfloat162*>(&xv[j]);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      ah[q] = __floats2bfloat162_rn(v[8 * j + 2 * q], v[8 * j + 2 * q + 1]);
-      const float2 af = __bfloat1622float2(ah[q]);
-      const float2 xf = __bfloat1622float2(xh[q]);
-      uh[q] = __floats2bfloat162_rn(fmaf(gg[2 * q], af.x, xf.x), fmaf(gg[2 * q + 1], af.y, xf.y));
-    }
-    reinterpret_cast<uint4*>(a_dst)[j] = av;
-    reinterpret_cast<uint4*>(u_dst)[j] = uv;
-  }
-}
-
-__device__ __forceinline__ void load_x_chunk(const __nv_bfloat16* xr, uint4* xv) {
-#pragma unroll
-  for (int j = 0; j < 4; ++j) xv[j] = __ldg(reinterpret_cast<const uint4*>(xr) + j);
-}
-
-template <int BN, int MODE>
+template <int MODE>
 __global__ void __launch_bounds__(kPThreads, 1)
-    proj_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
-                   const ProjParams p) {
-  constexpr int kStage = kPABytes + BN * 128;
-  constexpr bool kRes = MODE == kProjResidual || MODE == kProjResidualGated;
-  extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full_bar[8];
-  __shared__ __align__(8) uint64_t empty_bar[8];
-  __shared__ __align__(8) uint64_t acc_bar;
+    proj_tc_kernel(const __grid_constant__ ProjMaps maps, const ProjParams p) {
+  constexpr bool kRes = MODE != kProjQKV;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ __align__(8) uint64_t full_bar[kMaxStages];  // leader's: the stage's bytes of both CTAs
+  __shared__ __align__(8) uint64_t empty_bar[kMaxStages];
+  __shared__ __align__(8) uint64_t tfull_bar[2];
+  __shared__ __align__(8) uint64_t tempty_bar[2];         // leader's: the epilogue warps of both CTAs
   __shared__ __align__(8) uint64_t drain_bar;
   __shared__ uint32_t tmem_sh;
   __shared__ volatile int abort_flag;
-  __shared__ float s_bias[BN];
 
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* epi = smem + p.nst * kStage;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * kPM;
+  const uint32_t rank = cluster_rank();
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
-    for (int s = 0; s < p.nst; ++s) {
+    for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(smem_u32(&full_bar[s]), 1);
       mbar_init(smem_u32(&empty_bar[s]), 1);
     }
-    mbar_init(smem_u32(&acc_bar), 1);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(smem_u32(&tfull_bar[s]), 1);
+      mbar_init(smem_u32(&tempty_bar[s]), 2 * kEpiWarps);
+    }
     mbar_init(smem_u32(&drain_bar), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&amap)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&bmap)) : "memory");
   }
-  pdl_entry();
-  const int M = p.m_dev ? min(*reinterpret_cast<const volatile int*>(p.m_dev), p.M) : p.M;
-  if (p.row_stat && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
-    atomicAdd(p.row_stat, static_cast<unsigned long long>(M));
-  if (m0 >= M) return;  // uniform over the CTA, before TMEM is taken
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_sh)),
-                 "r"(BN < 32 ? 32 : BN)
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_sh)),
+                 "r"(kTmemCols)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     tc_fence_before();
   }
-  __syncthreads();
+  if (warp == 2 && lane <= kBoxes) {
+    const CUtensorMap* t = lane ? &maps.act[lane - 1] : &maps.w;
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(t)) : "memory");
+  }
+  cluster_arrive();
+  cluster_wait();  // both CTAs' barriers are initialised, TMEM is allocated
   tc_fence_after();
+  pdl_entry();
+  const int M = p.m_dev ? min(*reinterpret_cast<const volatile int*>(p.m_dev), p.M) : p.M;
+  if (p.row_stat && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(p.row_stat, static_cast<unsigned long long>(M));
   const uint32_t tmem = tmem_sh;
-  const int KB = p.K / 64;
-  const int nst = p.nst;
-  int issued = 0;  // producer: stages issued
+  const int nw = (p.N + 2 * kBM - 1) / (2 * kBM);
+  const int n = token_width(M, nw, n_pairs), half = n >> 1;
+  const int units = (M + n - 1) / n * nw;
+  const int sub = p.K / kBK, ks = (sub + kSub - 1) / kSub;
+  const int slot_bytes = kSub * (kABytes + half * (kBK * 2));
+  const int nst = min(kMaxStages, kRingBytes / slot_bytes);
+  const uint32_t ring = smem_u32(smem), ring_end = ring + nst * slot_bytes;
+  const uint32_t empty0 = smem_u32(&empty_bar[0]);
 
-  if (warp == 0) {
+  if (warp == 0 || warp == kTokWarp) {
     if (lane == 0) {
-      for (int kb = 0; kb < KB; ++kb) {
-        const int s = kb % nst;
-        if (kb >= nst && !mbar_wait(smem_u32(&empty_bar[s]), ((kb / nst) & 1) ^ 1, &abort_flag)) {
-          if (!abort_flag) report_status(p.status, kStatusWaitTimeout, 600);
-          abort_flag = 1;
-          break;
+      // ---------------- TMA producers: weights (warp 0), tokens ----------------
+      const bool wts = warp == 0;
+      const CUtensorMap* map = wts ? &maps.w : &maps.act[(n >> 5) - 1];
+      const uint32_t first = ring + (wts ? 0 : kSub * kABytes), end = first + nst * slot_bytes;
+      const uint32_t full0 = cluster_addr(smem_u32(&full_bar[0]), 0);
+      uint32_t dst = first, eb = empty0, fb = full0, par = 1u;
+      int issued = 0;
+      bool ok = true;
+      for (int u = pair; u < units && ok; u += n_pairs) {
+        const int tt = u / nw, w = u - tt * nw;
+        const int feat = w * 2 * kBM + static_cast<int>(rank) * kBM;
+        const int row = wts ? feat : tt * n + static_cast<int>(rank) * half;
+        const bool live = !wts || feat < p.N;  // this CTA's half of the weight tile has rows
+        // Bytes a stage brings into both CTAs (sub-blocks past the last are zero-filled).
+        const uint32_t tx = kSub * (kABytes * (w * 2 * kBM + kBM < p.N ? 2 : 1) + n * (kBK * 2));
+        for (int k = 0; k < ks; ++k) {
+          // The slot is free in both CTAs once the MMAs that read it are done;
+          // the leader arms its barrier with the bytes of both CTAs.
+          if (!(ok = mbar_wait_hot(eb, par, &abort_flag))) break;
+          if (wts && rank == 0) mbar_expect_tx(fb, tx);
+          if (live) tma_load_k64_pair(dst, map, row, k * kSub, fb);
+          ++issued;
+          dst += slot_bytes;
+          eb += 8;
+          fb += 8;
+          if (dst == end) {
+            dst = first;
+            eb = empty0;
+            fb = full0;
+            par ^= 1u;
+          }
         }
-        const uint32_t sa = smem_u32(smem + s * kStage);
-        mbar_expect_tx(smem_u32(&full_bar[s]), kStage);
-        tma_load_2d(sa, &amap, kb * 64, m0, smem_u32(&full_bar[s]));
-        tma_load_2d(sa + kPABytes, &bmap, kb * 64, n0, smem_u32(&full_bar[s]));
-        ++issued;
+      }
+      if (!ok) {
+        if (!abort_flag) report_status(p.status, kStatusWaitTimeout, wts ? 600 : 603);
+        abort_flag = 1;
+        // Copies already issued land before the CTAs can exit: the newest use
+        // of every slot (the leader's barriers see both CTAs').
+        for (int q = 0; wts && rank == 0 && q < nst && q < issued; ++q) {
+          const int last = issued - 1 - (issued - 1 - q) % nst;
+          const unsigned long long t0 = globaltimer();
+          while (!mbar_try(smem_u32(&full_bar[q]), (last / nst) & 1) && globaltimer() - t0 < kTcWaitNs) {
+          }
+        }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = instr_desc(kPM, BN);
+    if (lane == 0 && rank == 0) {
+      // ---------------- MMA issuer (the leader, for both CTAs) ----------------
+      const uint32_t w_lo0 = ((ring & 0x3FFFFu) >> 4) | (1u << 16), slot_lo = static_cast<uint32_t>(slot_bytes) >> 4;
+      const uint32_t w_end = ((ring_end & 0x3FFFFu) >> 4) | (1u << 16);
+      const uint32_t full0 = smem_u32(&full_bar[0]);
+      const uint32_t idesc = instr_desc(2 * kBM, n), b_sub = n * kBK >> 4;
+      uint32_t w_lo = w_lo0, fb = full0, eb = empty0, par = 0u, acc_phase = 0;
+      int acc = 0;
       bool ok = true;
-      for (int kb = 0; kb < KB; ++kb) {
-        const int s = kb % nst;
-        if (!mbar_wait(smem_u32(&full_bar[s]), (kb / nst) & 1, &abort_flag)) {
-          ok = false;
-          break;
-        }
+      for (int u = pair; u < units; u += n_pairs) {
+        if (!(ok = mbar_wait(smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, &abort_flag))) break;
         tc_fence_after();
-        const uint32_t sa = smem_u32(smem + s * kStage);
-        const uint32_t sb = sa + kPABytes;
+        const uint32_t d_tmem = tmem + static_cast<uint32_t>(acc * kMaxN);
+        for (int k = 0; k < ks; ++k) {
+          if (!(ok = mbar_wait_hot(fb, par, &abort_flag))) break;
+          tc_fence_after();
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
-          mma_bf16(tmem, smem_desc(sa + kk * 32), smem_desc(sb + kk * 32), idesc, (kb | kk) != 0);
-        mma_commit(smem_u32(&empty_bar[s]));
+          for (int q = 0; q < kSub; ++q) {
+            if (q && k * kSub + q >= sub) break;
+            const uint32_t wq = w_lo + q * (kABytes >> 4), xq = w_lo + (kSub * kABytes >> 4) + q * b_sub;
+#pragma unroll
+            for (int kk = 0; kk < kBK / 16; ++kk)
+              mma_bf16_pair(d_tmem, wq + kk * 2, xq + kk * 2, idesc, k != 0 || q != 0 || kk != 0);
+          }
+          mma_commit_pair(eb);
+          w_lo += slot_lo;
+          fb += 8;
+          eb += 8;
+          if (w_lo == w_end) {
+            w_lo = w_lo0;
+            fb = full0;
+            eb = empty0;
+            par ^= 1u;
+          }
+        }
+        if (!ok) break;
+        mma_commit_pair(smem_u32(&tfull_bar[acc]));
+        if (++acc == 2) {
+          acc = 0;
+          acc_phase ^= 1u;
+        }
       }
-      if (ok) {
-        mma_commit(smem_u32(&acc_bar));
-      } else {
+      if (!ok) {
         if (!abort_flag) report_status(p.status, kStatusWaitTimeout, 601);
         abort_flag = 1;
       }
       // Every MMA issued so far has completed once the drain barrier fires.
-      mma_commit(smem_u32(&drain_bar));
+      mma_commit_pair(smem_u32(&drain_bar));
       const unsigned long long t0 = globaltimer();
       while (!mbar_try(smem_u32(&drain_bar), 0) && globaltimer() - t0 < kTcWaitNs) {
       }
     }
   } else {
-    const int quad = warp & 3;
-    const int r = quad * 32 + lane;
-    const int m = m0 + r;
-    uint8_t* stage = epi + (warp - 2) * kPEpiStage;
-    // While the MMAs run: the tile's bias into shared memory, this lane's
-    // row pointers, and the residual rows' first chunk of x.
-    for (int j = threadIdx.x - 64; j < BN; j += 128) s_bias[j] = p.bias ? __ldg(p.bias + n0 + j) : 0.f;
-    __nv_bfloat16* dst = nullptr;
-    const __nv_bfloat16* xr = nullptr;
-    __nv_bfloat16* ur = nullptr;
-    __nv_bfloat16* gr[kMaxRowOf];
+    // ---------------- Epilogue ----------------
+    const int quad = warp & 3;           // TMEM lanes [32 quad, 32 quad + 32)
+    const int part = (warp - 2) >> 2;    // which half of the tile's token columns
+    uint32_t* stage = reinterpret_cast<uint32_t*>(smem + kRingBytes + (warp - 2) * kStageOut);
+    const uint32_t tempty0 = cluster_addr(smem_u32(&tempty_bar[0]), 0);
+    const int s_row = lane >> 2, s_ch = lane & 3;  // this lane's row (of 8) and 16-byte chunk of a staged store
+    int acc = 0;
+    uint32_t acc_phase = 0;
+    bool ok = true;
+    for (int u = pair; u < units; u += n_pairs) {
+      const int tt = u / nw, w = u - tt * nw;
+      const int feat = w * 2 * kBM + static_cast<int>(rank) * kBM + quad * 32;  // the warp's 32 features
+      const int m0 = tt * n;
+      const int c_lo = part * half, c_hi = feat < p.N ? min(c_lo + half, M - m0) : 0;
+      const float bias = p.bias && feat < p.N ? __ldg(p.bias + feat + lane) : 0.f;
+      if (!(ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&tfull_bar[acc]), acc_phase, &abort_flag)))) break;
+      tc_fence_after();
+      const uint32_t tb = tmem + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(acc * kMaxN);
+#pragma unroll 1
+      for (int c = c_lo; c < c_hi; c += 32) {
+        // This lane's token of the chunk (c + lane) and the row its values go to.
+        const int m = m0 + c + lane;
+        int row = -1;
+        if (c + lane < c_hi) {
+          if constexpr (kRes) {
+            row = p.rows ? p.rows[m] : m;
+            if (row < 0 || row >= p.n_tok) {
+              report_status(p.status, kStatusBadIndex, 6000000 + m);
+              row = -1;
+            }
+          } else {
+            row = m;
+          }
+        }
+        uint32_t v[32];
+        tmem_ld32_async(tb + c, v);
+        if constexpr (kRes) {
+          // The residual input rows in the staged stores' layout, in flight
+          // while the tile is read and staged.
+          uint4 xv[4];
+          int tok[4];
 #pragma unroll
-    for (int q = 0; q < kMaxRowOf; ++q) gr[q] = nullptr;
-    const int n_g = p.row_of ? p.row_w : 0;
-    __nv_bfloat16* krow = nullptr;  // kProjQKV: this lane's k row (dst holds its q row)
-    const float* grow = nullptr;    // kProjResidualGated: this lane's gate row
-    if (m < M) {
-      if constexpr (MODE == kProjStore) {
-        dst = p.out + static_cast<size_t>(m) * p.ldo + n0;
-      } else if constexpr (MODE == kProjQKV) {
-        const int qi = p.inv ? p.inv[m] : m;
-        const int Dm = p.N / 3;
-        if (qi >= 0) dst = p.q_out + static_cast<size_t>(qi) * Dm;
-        krow = p.k_out + static_cast<size_t>(m) * Dm;
-      } else {
-        const int t = p.rows ? p.rows[m] : m;
-        if (t >= 0 && t < p.n_tok) {
-          const size_t off = static_cast<size_t>(t) * p.N + n0;
-          dst = p.a_out + off;
-          xr = p.x + off;
-          ur = p.u_out + off;
-          if constexpr (MODE == kProjResidualGated) grow = p.gate + static_cast<size_t>(t / p.seq) * p.gate_ld + n0;
+          for (int it = 0; it < 4; ++it) {
+            tok[it] = __shfl_sync(0xffffffffu, row, it * 8 + s_row);
+            if (tok[it] >= 0)
+              xv[it] = __ldg(reinterpret_cast<const uint4*>(p.x + static_cast<size_t>(tok[it]) * p.N + feat + s_ch * 8));
+          }
+          tmem_wait32(v);
+          __syncwarp();
+          stage_by_token(stage, v, bias, lane);
+          __syncwarp();
 #pragma unroll
-          for (int q = 0; q < kMaxRowOf; ++q) {
-            if (q < n_g) {
-              const int pos = p.row_of[static_cast<size_t>(t) * p.row_w + q];
-              if (pos >= 0) gr[q] = p.xg + static_cast<size_t>(pos) * p.N + n0;
+          for (int it = 0; it < 4; ++it) {
+            const uint4 av = *reinterpret_cast<const uint4*>(stage + (it * 8 + s_row) * 16 + s_ch * 4);
+            if (tok[it] < 0) continue;
+            const size_t off = static_cast<size_t>(tok[it]) * p.N + feat + s_ch * 8;
+            float gg[8];
+            if constexpr (MODE == kProjResidualGated) {
+              const float* g = p.gate + static_cast<size_t>(tok[it] / p.seq) * p.gate_ld + feat + s_ch * 8;
+              const float4 g0 = __ldg(reinterpret_cast<const float4*>(g));
+              const float4 g1 = __ldg(reinterpret_cast<const float4*>(g) + 1);
+              gg[0] = g0.x; gg[1] = g0.y; gg[2] = g0.z; gg[3] = g0.w;
+              gg[4] = g1.x; gg[5] = g1.y; gg[6] = g1.z; gg[7] = g1.w;
+            }
+            uint4 uv;
+            const __nv_bfloat162* ah = reinterpret_cast<const __nv_bfloat162*>(&av);
+            const __nv_bfloat162* xh = reinterpret_cast<const __nv_bfloat162*>(&xv[it]);
+            __nv_bfloat162* uh = reinterpret_cast<__nv_bfloat162*>(&uv);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const float2 af = __bfloat1622float2(ah[q]), xf = __bfloat1622float2(xh[q]);
+              if constexpr (MODE == kProjResidualGated)
+                uh[q] = __floats2bfloat162_rn(fmaf(gg[2 * q], af.x, xf.x), fmaf(gg[2 * q + 1], af.y, xf.y));
+              else
+                uh[q] = __floats2bfloat162_rn(xf.x + af.x, xf.y + af.y);
+            }
+            *reinterpret_cast<uint4*>(p.a_out + off) = av;
+            *reinterpret_cast<uint4*>(p.u_out + off) = uv;
+            if constexpr (MODE == kProjResidual) {
+              const int n_g = p.row_of ? p.row_w : 0;
+              for (int q = 0; q < n_g; ++q) {
+                const int pos = __ldg(p.row_of + static_cast<size_t>(tok[it]) * p.row_w + q);
+                if (pos >= 0) *reinterpret_cast<uint4*>(p.xg + static_cast<size_t>(pos) * p.N + feat + s_ch * 8) = uv;
+              }
             }
           }
         } else {
-          report_status(p.status, kStatusBadIndex, 6000000 + m);
-        }
-      }
-    }
-    uint4 xb[2][4];  // residual mode: x of chunks c and c + 1 in flight
-    if constexpr (kRes) {
-      if (xr) {
-        load_x_chunk(xr, xb[0]);
-        if (BN > 32) load_x_chunk(xr + 32, xb[1]);
-      }
-    }
-    asm volatile("bar.sync 1, 128;" ::: "memory");  // the four epilogue warps: bias staged
-    if (mbar_wait(smem_u32(&acc_bar), 0, &abort_flag)) {
-      tc_fence_after();
-      const uint32_t tbase = tmem + (static_cast<uint32_t>(quad * 32) << 16);
-      if constexpr (kRes) {
+          // The warp's features lie in one of q, k, v (D is a multiple of 64).
+          const int Dm = p.N / 3, region = feat / Dm, f = feat - region * Dm;
+          if (region == 0 && row >= 0 && p.inv) row = p.inv[m];
+          tmem_wait32(v);
+          __syncwarp();
+          if (region < 2) {
+            stage_by_token(stage, v, bias, lane);
+            __syncwarp();
+            __nv_bfloat16* base = (region == 0 ? p.q_out : p.k_out) + f + s_ch * 8;
 #pragma unroll
-        for (int c = 0; c < BN / 32; ++c) {
-          uint4 xc[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) xc[j] = xb[c & 1][j];
-          if (xr && c + 2 < BN / 32) load_x_chunk(xr + (c + 2) * 32, xb[c & 1]);  // two chunks ahead
-          uint32_t raw[32];
-          tmem_ld32(tbase + c * 32, raw);
-          float v[32];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(raw[j]) + s_bias[c * 32 + j];
-          if (dst) {
-            if constexpr (MODE == kProjResidualGated) {
-              store_residual_gated(v, xc, grow + c * 32, dst + c * 32, ur + c * 32);
-            } else {
-              __nv_bfloat16* gc[kMaxRowOf];
-#pragma unroll
-              for (int q = 0; q < kMaxRowOf; ++q) gc[q] = gr[q] ? gr[q] + c * 32 : nullptr;
-              store_residual(v, xc, dst + c * 32, ur + c * 32, gc, n_g);
+            for (int it = 0; it < 4; ++it) {
+              const uint4 val = *reinterpret_cast<const uint4*>(stage + (it * 8 + s_row) * 16 + s_ch * 4);
+              const int r = __shfl_sync(0xffffffffu, row, it * 8 + s_row);
+              if (r >= 0) *reinterpret_cast<uint4*>(base + static_cast<size_t>(r) * Dm) = val;
             }
-          }
-        }
-      } else {
-        // Store-type epilogues stay rolled: the chunk body is large and an
-        // unrolled copy per chunk spills out of the instruction cache.
-#pragma unroll 1
-        for (int c = 0; c < BN / 32; ++c) {
-          uint32_t raw[32];
-          tmem_ld32(tbase + c * 32, raw);
-          float v[32];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(raw[j]) + s_bias[c * 32 + j];
-          if constexpr (MODE == kProjStore) {
-            store_chunk_staged(stage, v, dst ? dst + c * 32 : nullptr, lane);
           } else {
-            // The chunk lies in one of q, k, v (D is a multiple of 64): warp-uniform.
-            const int Dm = p.N / 3;
-            const int col = n0 + c * 32;
-            const int region = col / Dm, cc = col - region * Dm;
-            if (region == 0) {
-              store_chunk_staged(stage, v, dst ? dst + cc : nullptr, lane);
-            } else if (region == 1) {
-              store_chunk_staged(stage, v, krow ? krow + cc : nullptr, lane);
-            } else {
-              store_chunk_transposed(stage, v, p.vt_out + static_cast<size_t>(cc) * p.n_tok, m0 + quad * 32, M,
-                                     static_cast<size_t>(p.n_tok), lane);
+            // v^T: rows are features; 8 consecutive tokens per lane (the token
+            // count is a multiple of 8).
+            stage_by_feature(stage, v, bias, lane);
+            __syncwarp();
+            __nv_bfloat16* base = p.vt_out + static_cast<size_t>(f) * p.n_tok + m0 + c + s_ch * 8;
+#pragma unroll
+            for (int it = 0; it < 4; ++it) {
+              const int fr = it * 8 + s_row;
+              const uint4 val = reinterpret_cast<const uint4*>(stage)[fr * 4 + (s_ch ^ ((fr >> 1) & 3))];
+              if (c + s_ch * 8 < c_hi) *reinterpret_cast<uint4*>(base + static_cast<size_t>(fr) * p.n_tok) = val;
             }
           }
         }
       }
-    } else if (lane == 0) {
-      if (!abort_flag) report_status(p.status, kStatusWaitTimeout, 602);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(tempty0 + acc * 8);
+      if (++acc == 2) {
+        acc = 0;
+        acc_phase ^= 1u;
+      }
+    }
+    if (!ok) {
+      if (lane == 0 && !abort_flag) report_status(p.status, kStatusWaitTimeout, 602);
       abort_flag = 1;
     }
   }
+  // Neither CTA leaves (or frees TMEM) while the other may still reach its
+  // shared memory or the pair's MMAs run.
   tc_fence_before();
-  __syncthreads();
-  if (warp == 0 && lane == 0 && abort_flag) {
-    // Copies issued but never consumed still land in shared memory: wait for
-    // the newest phase of every stage before the CTA exits.
-    for (int s = 0; s < nst && s < issued; ++s) {
-      const int last = issued - 1 - ((issued - 1 - s) % nst);  // newest k-block issued on stage s
-      const unsigned long long t0 = globaltimer();
-      while (!mbar_try(smem_u32(&full_bar[s]), (last / nst) & 1) && globaltimer() - t0 < kTcWaitNs) {
-      }
-    }
-  }
-  __syncthreads();
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN < 32 ? 32 : BN)
-                 : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
   }
-}
-
-template <int BN>
-constexpr int stage_bytes() {
-  return kPABytes + BN * 128;
 }
 
 }  // namespace
 
-int proj_tile_n(int N, int want) {
-  if (want) return (want == 64 || want == 128 || want == 256) && N % want == 0 ? want : 0;
-  if (N % 256 == 0) return 256;
-  if (N % 128 == 0) return 128;
-  if (N % 64 == 0) return 64;
-  return 0;
-}
-
-cudaError_t launch_proj_tc(const ProjArgs& a, cudaStream_t s) {
-  const int BN = proj_tile_n(a.N, a.tile_n);
-  if (BN == 0 || a.K % 64 || a.M <= 0) return cudaErrorInvalidValue;
+cudaError_t launch_proj_tc(const ProjArgs& a, int n_sms, cudaStream_t s) {
+  if (a.N % 64 || a.K % 64 || a.M <= 0) return cudaErrorInvalidValue;
   if (a.mode == kProjResidualGated && (!a.gate || a.seq <= 0 || a.row_of)) return cudaErrorInvalidValue;
-  CUtensorMap amap, bmap;
-  if (!encode_2d(&amap, a.A, static_cast<uint64_t>(a.a_rows), static_cast<uint64_t>(a.K), kPM) ||
-      !encode_2d(&bmap, a.B, static_cast<uint64_t>(a.N), static_cast<uint64_t>(a.K), static_cast<uint32_t>(BN)))
+  ProjMaps maps;
+  if (!encode_k64(&maps.w, a.B, static_cast<uint64_t>(a.N), static_cast<uint64_t>(a.K), kBM, kSub))
     return cudaErrorInvalidValue;
+  for (int i = 0; i < kBoxes; ++i)
+    if (!encode_k64(&maps.act[i], a.A, static_cast<uint64_t>(a.a_rows), static_cast<uint64_t>(a.K), 16 * (i + 1), kSub))
+      return cudaErrorInvalidValue;
   ProjParams p{};
-  p.M = a.M; p.N = a.N; p.K = a.K; p.m_dev = a.m_dev; p.bias = a.bias; p.mode = a.mode;
-  p.out = static_cast<__nv_bfloat16*>(a.out); p.ldo = a.ldo;
+  p.M = a.M; p.N = a.N; p.K = a.K; p.m_dev = a.m_dev; p.bias = a.bias;
   p.rows = a.rows; p.n_tok = a.n_tok;
   p.x = static_cast<const __nv_bfloat16*>(a.x);
   p.a_out = static_cast<__nv_bfloat16*>(a.a_out);
@@ -456,33 +476,19 @@ cudaError_t launch_proj_tc(const ProjArgs& a, cudaStream_t s) {
   p.vt_out = static_cast<__nv_bfloat16*>(a.vt_out);
   p.gate = a.gate; p.gate_ld = a.gate_ld; p.seq = a.seq;
   p.status = a.status;
-  const int kb = a.K / 64;
-  const int stage = kPABytes + BN * 128;
-  int nst = (200 * 1024) / stage;
-  nst = nst > 8 ? 8 : nst;
-  nst = nst > kb ? kb : nst;
-  if (nst < 1) nst = 1;
-  p.nst = nst;
-  const size_t smem = static_cast<size_t>(nst) * stage + 4 * kPEpiStage + 1024;
-  const dim3 grid(a.N / BN, (a.M + kPM - 1) / kPM);
+  // At most one pair per tile of the narrowest width.
+  const int nw = (a.N + 2 * kBM - 1) / (2 * kBM);
+  const int pairs = std::max(1, std::min(n_sms / 2, (a.M + 31) / 32 * nw));
   auto run = [&](auto kern) -> cudaError_t {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const cudaError_t e = set_dyn_smem_on_device(reinterpret_cast<const void*>(kern), kPSmem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(kern, grid, dim3(kPThreads), smem, s, amap, bmap, p);
+    return launch_pdl<2>(kern, dim3(2 * pairs), dim3(kPThreads), kPSmem, s, maps, p);
   };
-  auto by_mode = [&](auto bn) -> cudaError_t {
-    constexpr int kBN = decltype(bn)::value;
-    switch (a.mode) {
-      case kProjQKV: return run(proj_tc_kernel<kBN, kProjQKV>);
-      case kProjResidual: return run(proj_tc_kernel<kBN, kProjResidual>);
-      case kProjResidualGated: return run(proj_tc_kernel<kBN, kProjResidualGated>);
-      default: return run(proj_tc_kernel<kBN, kProjStore>);
-    }
-  };
-  switch (BN) {
-    case 256: return by_mode(std::integral_constant<int, 256>{});
-    case 128: return by_mode(std::integral_constant<int, 128>{});
-    default: return by_mode(std::integral_constant<int, 64>{});
+  switch (a.mode) {
+    case kProjQKV: return run(proj_tc_kernel<kProjQKV>);
+    case kProjResidual: return run(proj_tc_kernel<kProjResidual>);
+    case kProjResidualGated: return run(proj_tc_kernel<kProjResidualGated>);
+    default: return cudaErrorInvalidValue;
   }
 }
 
