@@ -85,7 +85,6 @@ __global__ void __launch_bounds__(kModWarps * 32) ada_mod_kernel(AdaModArgs a) {
 }
 
 constexpr int kLnWarps = 8;
-constexpr int kLnChunks = kAdaLnMaxD / 256;  // 16-byte chunks per lane
 
 // Eight floats from global or shared memory (a generic pointer: the row
 // pass reads the modulation vectors from either).
@@ -119,11 +118,12 @@ __device__ __forceinline__ uint4 pack8(const float* f) {
 
 // Mean and 1 / sqrt(var + eps) of the row held as bf16 chunks (chunk c = lane + 32 q),
 // two passes over the registers.
+template <int C>
 __device__ __forceinline__ void row_stats(const uint4* v, int nvec, int lane, int D, float eps, float& mean,
                                           float& rstd) {
   float s = 0.f;
 #pragma unroll
-  for (int q = 0; q < kLnChunks; ++q) {
+  for (int q = 0; q < C; ++q) {
     if (lane + 32 * q < nvec) {
       float f[8];
       unpack_vec(v[q], f, static_cast<__nv_bfloat16*>(nullptr));
@@ -134,7 +134,7 @@ __device__ __forceinline__ void row_stats(const uint4* v, int nvec, int lane, in
   mean = warp_sum(s) / static_cast<float>(D);
   float ss = 0.f;
 #pragma unroll
-  for (int q = 0; q < kLnChunks; ++q) {
+  for (int q = 0; q < C; ++q) {
     if (lane + 32 * q < nvec) {
       float f[8];
       unpack_vec(v[q], f, static_cast<__nv_bfloat16*>(nullptr));
@@ -149,11 +149,12 @@ __device__ __forceinline__ void row_stats(const uint4* v, int nvec, int lane, in
 }
 
 // dst = bf16((v - mean) rstd (1 + scale) + shift), chunk by chunk.
+template <int C>
 __device__ __forceinline__ void store_modulated(const uint4* v, int nvec, int lane, float mean, float rstd,
                                                 const float* shift, const float* scale, __nv_bfloat16* dst,
                                                 __nv_bfloat16* dst2) {
 #pragma unroll
-  for (int q = 0; q < kLnChunks; ++q) {
+  for (int q = 0; q < C; ++q) {
     const int c = lane + 32 * q;
     if (c < nvec) {
       float f[8], sh[8], sc[8];
@@ -173,6 +174,12 @@ __device__ __forceinline__ void store_modulated(const uint4* v, int nvec, int la
 // one sample (seq is a multiple of 8): the block stages that sample's first
 // five vectors (shift_a .. scale_m, 5D floats) in shared memory, loaded
 // together with the rows.  A listed-row launch reads them from L2 per row.
+// C bounds a lane's 16-byte chunks of a row, ceil(D / 256): a kernel for the
+// widest row only (10 chunks, 3 of them used at D 768) spent most of its
+// instructions and registers on the absent ones: an AdaLN sampler pass of 4
+// steps with 8 row launches went from 602 to 587 us with the bound (D 768,
+// 2048 tokens).
+template <int C>
 __global__ void __launch_bounds__(kLnWarps * 32) adaln_rows_kernel(AdaLnArgs a) {
   extern __shared__ __align__(16) float s_mod[];  // [5, D] when staged
   pdl_entry();
@@ -190,18 +197,18 @@ __global__ void __launch_bounds__(kLnWarps * 32) adaln_rows_kernel(AdaLnArgs a) 
     }
   }
   const size_t off = static_cast<size_t>(t < 0 ? 0 : t) * D;
-  uint4 v[kLnChunks], av[kLnChunks];
+  uint4 v[C], av[C];
   const uint4* a4 =
       a.a ? reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(a.a) + off) : nullptr;
   if (t >= 0 && (a.h_out || a4)) {
     // x and the cached attention row in flight together (and with the staging below).
     const uint4* x4 = reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(a.x) + off);
 #pragma unroll
-    for (int q = 0; q < kLnChunks; ++q)
+    for (int q = 0; q < C; ++q)
       if (lane + 32 * q < nvec) v[q] = x4[lane + 32 * q];
     if (a4) {
 #pragma unroll
-      for (int q = 0; q < kLnChunks; ++q)
+      for (int q = 0; q < C; ++q)
         if (lane + 32 * q < nvec) av[q] = a4[lane + 32 * q];
     }
   }
@@ -219,13 +226,13 @@ __global__ void __launch_bounds__(kLnWarps * 32) adaln_rows_kernel(AdaLnArgs a) 
   __nv_bfloat16* u = static_cast<__nv_bfloat16*>(a.u) + off;
   float mean, rstd;
   if (a.h_out) {
-    row_stats(v, nvec, lane, D, a.eps, mean, rstd);
-    store_modulated(v, nvec, lane, mean, rstd, md, md + D, static_cast<__nv_bfloat16*>(a.h_out) + off, nullptr);
+    row_stats<C>(v, nvec, lane, D, a.eps, mean, rstd);
+    store_modulated<C>(v, nvec, lane, mean, rstd, md, md + D, static_cast<__nv_bfloat16*>(a.h_out) + off, nullptr);
   }
   if (a4) {
     // u = bf16(x + gate_a a): one rounding of the fused product-sum.
 #pragma unroll
-    for (int q = 0; q < kLnChunks; ++q) {
+    for (int q = 0; q < C; ++q) {
       const int c = lane + 32 * q;
       if (c < nvec) {
         float xf[8], af[8], g[8];
@@ -240,12 +247,12 @@ __global__ void __launch_bounds__(kLnWarps * 32) adaln_rows_kernel(AdaLnArgs a) 
     }
   } else if (a.m_out) {
 #pragma unroll
-    for (int q = 0; q < kLnChunks; ++q)
+    for (int q = 0; q < C; ++q)
       if (lane + 32 * q < nvec) v[q] = reinterpret_cast<const uint4*>(u)[lane + 32 * q];
   }
   if (a.m_out) {
-    row_stats(v, nvec, lane, D, a.eps, mean, rstd);
-    store_modulated(v, nvec, lane, mean, rstd, md + 3 * D, md + 4 * D,
+    row_stats<C>(v, nvec, lane, D, a.eps, mean, rstd);
+    store_modulated<C>(v, nvec, lane, mean, rstd, md + 3 * D, md + 4 * D,
                     static_cast<__nv_bfloat16*>(a.m_out) + off,
                     a.m_copy ? static_cast<__nv_bfloat16*>(a.m_copy) + off : nullptr);
   }
@@ -316,12 +323,21 @@ cudaError_t launch_adaln_rows(const AdaLnArgs& a, cudaStream_t s) {
   if (a.seq <= 0 || a.D % 64 || a.D > kAdaLnMaxD) return cudaErrorInvalidValue;
   const int grid = (a.T + kLnWarps - 1) / kLnWarps;
   const size_t smem = a.rows ? 0 : static_cast<size_t>(5) * a.D * sizeof(float);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(adaln_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-  }
-  return launch_pdl(adaln_rows_kernel, dim3(grid), dim3(kLnWarps * 32), smem, s, a);
+  auto run = [&](auto kern) -> cudaError_t {
+    if (smem > 48 * 1024) {
+      const cudaError_t e = set_dyn_smem_on_device(reinterpret_cast<const void*>(kern), static_cast<int>(smem));
+      if (e != cudaSuccess) return e;
+    }
+    return launch_pdl(kern, dim3(grid), dim3(kLnWarps * 32), smem, s, a);
+  };
+  const int chunks = (a.D + 255) / 256;
+  if (chunks <= 2) return run(adaln_rows_kernel<2>);
+  if (chunks == 3) return run(adaln_rows_kernel<3>);
+  if (chunks == 4) return run(adaln_rows_kernel<4>);
+  if (chunks == 5) return run(adaln_rows_kernel<5>);
+  if (chunks <= 7) return run(adaln_rows_kernel<7>);
+  static_assert(kAdaLnMaxD <= 10 * 256, "chunks per lane");
+  return run(adaln_rows_kernel<10>);
 }
 
 cudaError_t launch_ddpm(const DdpmArgs& a, cudaStream_t s) {
