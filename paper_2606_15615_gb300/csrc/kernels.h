@@ -97,6 +97,22 @@ cudaError_t launch_compact(const CompactArgs& a, bool bf16, cudaStream_t s);
 // gather_kernel alone: the listed rows of a.x into a.xg (lists already built).
 cudaError_t launch_gather(const CompactArgs& a, bool bf16, cudaStream_t s);
 
+// select, compact and gather in one launch, with an exchange of the blocks' row
+// counts between them.
+struct DecideArgs {
+  SelectArgs sel;             // block_counts, block_offsets and done are not used
+  int32_t* list;              // [rows]
+  const void* x;              // [T, D]
+  void* xg;                   // [rows, D] gathered inputs, or null: gathered later (launch_gather)
+  int row_vecs;               // 16-byte vectors of a row
+  unsigned long long* words;  // [blocks, G] tagged row counts
+  unsigned* epoch;            // tag of the last launch over these words, 0 before the first
+};
+// Blocks of a launch over max_tokens tokens when they are all resident at
+// once, which the exchange needs; 0 when they are not (the three kernels).
+int decide_blocks(int max_tokens, int k, int n_sms);
+cudaError_t launch_decide(const DecideArgs& a, cudaStream_t s);
+
 // Grouped expert FFN over the compacted rows (Eq. 5 / Eq. 6 on R only).
 struct FfnArgs {
   int G, E, D, F, k, T;

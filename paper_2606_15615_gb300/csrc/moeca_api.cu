@@ -124,6 +124,7 @@ struct moeca_handle {
   int* tc_work = nullptr;       // GEMM unit tickets {next, CTAs done}, left at 0
   int tc_dep_pairs_n = 0;
   PrepShape prep{0, 0, 0, 0, false};  // fused router + select + compact, when it fits
+  int decide_blocks = 0;        // separate path: decide_kernel's blocks at max_tokens (0: the three kernels)
   unsigned prep_epoch = 0;      // tag of the last fused launch (its exchanges' words)
   bool inject_stall = false;    // moeca_inject_fault: next step's exchanges wait for a tag nobody writes
   unsigned long long* prep_words = nullptr;  // tagged exchange words: partials, then row counts
@@ -553,6 +554,7 @@ moeca_status moeca_create(const moeca_config* cfg, const moeca_layer_weights* la
     A((void**)&h->attn_inv, T * 4);
     A((void**)&h->attn_rowof, T * (k + c.n_shared) * 4);
   }
+  bool separate = true;  // router, then decide (or select, compact, gather)
   const size_t nblk_router = (T + kRouterTokensPerBlock - 1) / kRouterTokensPerBlock;
   const size_t nblk_sel = (T + kSelectTokensPerBlock - 1) / kSelectTokensPerBlock;
   A((void**)&h->partials, nblk_router * E * 2 * 4);
@@ -587,7 +589,14 @@ moeca_status moeca_create(const moeca_config* cfg, const moeca_layer_weights* la
       h->prep_count_off = nb * E * 2;
       h->prep_words_n = h->prep_count_off + nb * (G + 1);
       A((void**)&h->prep_words, h->prep_words_n * 8);
+      separate = false;
     }
+  }
+  if (separate) {
+    h->decide_blocks = decide_blocks(c.max_tokens, c.top_k, h->n_sms);
+    // The words, then the last launch's tag.
+    h->prep_words_n = h->decide_blocks ? static_cast<size_t>(h->decide_blocks) * G + 1 : 0;
+    if (h->decide_blocks) A((void**)&h->prep_words, h->prep_words_n * 8);
   }
   h->act.assign(c.n_layers, nullptr);
   for (int l = 1; l < c.n_layers && ok; ++l) A(&h->act[l], T * D * es);
@@ -810,6 +819,17 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
       if ((e = timed(h, MOECA_K_PREP, s, [&] { return launch_prep(pa, h->prep, s); })) != cudaSuccess) break;
     } else {
       if ((e = timed(h, MOECA_K_ROUTER, s, [&] { return launch_router(ra, h->bf16, s); })) != cudaSuccess) break;
+      if (h->decide_blocks) {
+        DecideArgs da{};
+        da.sel = sa; da.list = L.list; da.x = moe_in; da.xg = xg_now;
+        da.row_vecs = static_cast<int>(c.hidden * h->es / 16);
+        da.words = h->prep_words;
+        da.epoch = reinterpret_cast<unsigned*>(h->prep_words + h->prep_words_n - 1);
+        e = timed(h, MOECA_K_SELECT, s, [&] { return launch_decide(da, s); });
+        if (e != cudaSuccess) break;
+      }
+    }
+    if (!fused && !h->decide_blocks) {
       if ((e = timed(h, MOECA_K_SELECT, s, [&] { return launch_select(sa, s); })) != cudaSuccess) break;
       if ((e = timed(h, MOECA_K_COMPACT, s, [&] { return launch_compact(ca, h->bf16, s); })) != cudaSuccess) break;
     }

@@ -17,7 +17,13 @@
 // list (token * k + slot for routed experts, token for the shared expert).
 // gather_kernel then copies every listed row's layer input into a
 // contiguous buffer for the GEMMs, one warp per row over the whole list.
+//
+// decide_kernel does all of it in one launch while its grid of 32-token blocks
+// is co-resident (decide_blocks): decisions, an exchange of the blocks' row
+// counts, row lists and row gather, as the fused preparation kernel does after
+// its thresholds.  The three kernels above take larger token counts.
 #include "common.cuh"
+#include "exchange.cuh"
 #include "kernels.h"
 #include "select_token.cuh"
 
@@ -241,7 +247,232 @@ __global__ void __launch_bounds__(256) gather_kernel(CompactArgs a) {
   }
 }
 
+// ---- select, compact and gather in one launch ----
+// The three kernels are latency, not bytes: each starts, waits on a chain of
+// loads and ends, with 128 tokens in a block (32 blocks at 4096 tokens), and
+// the gather reads a token's row once per recomputed branch.  Here one warp of
+// a 32-token block decides a token per lane, the blocks exchange their row
+// counts per group as tagged words, and every warp copies its tokens' rows,
+// each read once and written to all its places.  Event-timed, three kernels ->
+// this one, full / cache step: 64 experts top-8 at 4096 tokens, D 1152
+// 42 -> 26 / 36 -> 22 us; D 2560, 4 + 1 experts 29 -> 22 / 25 -> 19 us; fp32,
+// D 384, 512 tokens 18 -> 12 us.
+constexpr int kDecTokens = 32;
+constexpr int kDecThreads = 256;
+constexpr unsigned long long kDecWaitNs = 1000000000ull;
+
+template <int KMAX>
+__global__ void __launch_bounds__(kDecThreads) decide_kernel(DecideArgs a) {
+  __shared__ int32_t s_re[kDecTokens * KMAX], s_ce[kDecTokens * KMAX];
+  __shared__ float s_rw[kDecTokens * KMAX], s_cw[kDecTokens * KMAX], s_cn[kDecTokens * KMAX];
+  __shared__ float s_tau[kMaxExperts];
+  __shared__ unsigned s_bal[kMaxGroups];
+  __shared__ int s_part[kDecThreads][2];
+  __shared__ int s_pre[kMaxGroups], s_tot[kMaxGroups], s_off[kMaxGroups + 1];
+  __shared__ int s_pos[kDecTokens][KMAX + 1];  // list position of each of a token's rows, -1: none
+  __shared__ int s_fail;
+  const SelectArgs& sel = a.sel;
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int k = sel.k, E = sel.E, G = sel.G;
+  const int tok0 = blockIdx.x * kDecTokens, ntok = min(kDecTokens, sel.T - tok0);
+  const size_t b0 = static_cast<size_t>(tok0) * k;
+  // Before the dependency wait: the cached metadata.  The previous kernel is
+  // this layer's router, which passed its own wait, so the kernels that wrote
+  // them (this one and the combine, a step earlier) have ended.
+  if (!sel.refresh)
+    for (int idx = t; idx < ntok * k; idx += kDecThreads) {
+      s_ce[idx] = sel.cache_e[b0 + idx];
+      s_cw[idx] = sel.cache_w[b0 + idx];
+      s_cn[idx] = sel.cache_norm[b0 + idx];
+    }
+  if (t == 0) s_fail = 0;
+  pdl_entry();
+  // This launch's tag: one past the last launch's, kept on the device (a
+  // captured launch can be replayed), and advanced by block 0 once it has read
+  // every block's words, so every block has read it.
+  unsigned epoch = *a.epoch + 1;
+  if (epoch == 0) epoch = 1;  // 0 marks words never written
+  for (int idx = t; idx < ntok * k; idx += kDecThreads) {
+    s_re[idx] = sel.route_e[b0 + idx];
+    s_rw[idx] = sel.route_w[b0 + idx];
+  }
+  if (t < E) s_tau[t] = sel.tau[t];
+  __syncthreads();
+
+  TokenDecisionT<KMAX> d;
+  if (warp == 0) {
+    const bool valid = lane < ntok;
+    const int q = valid ? lane * k : 0;
+    TokenPrepT<KMAX> tp;
+    prepare_token(sel, tok0 + lane, valid, s_re + q, s_rw + q, s_ce + q, s_cw + q, s_cn + q, tp);
+    finish_token(sel, tok0 + lane, tp, s_tau, d);
+    // Groups in which this lane's token has a row.
+    uint32_t gm[3] = {0u, 0u, 0u};
+#pragma unroll
+    for (int p = 0; p < KMAX; ++p)
+      if (d.rec[p]) gm[d.e[p] >> 5] |= 1u << (d.e[p] & 31);
+    if (d.shared_row) gm[E >> 5] |= 1u << (E & 31);
+    for (int g = 0; g < G; ++g) {
+      const unsigned b = __ballot_sync(0xffffffffu, (gm[g >> 5] >> (g & 31)) & 1u);
+      if (lane == (g & 31)) s_bal[g] = b;
+    }
+    __syncwarp();
+    for (int g = lane; g < G; g += 32)
+      st_word(a.words + static_cast<size_t>(blockIdx.x) * G + g, tag_word(__popc(s_bal[g]), epoch));
+    const int c_matched = warp_sum_i(d.n_matched), c_rec = warp_sum_i(d.n_rec), c_near = warp_sum_i(d.n_near);
+    const int c_full = warp_sum_i(valid && !d.bad && !d.any ? 1 : 0), c_shared = warp_sum_i(d.shared_row ? 1 : 0);
+    if (lane == 0) {
+      unsigned long long* st = sel.stats;
+      atomicAdd(st + kStRecomputed, static_cast<unsigned long long>(c_rec));
+      atomicAdd(st + kStReused, static_cast<unsigned long long>(ntok * k - c_rec));
+      if (c_shared) atomicAdd(st + kStSharedRecomputed, static_cast<unsigned long long>(c_shared));
+      if (!sel.refresh) {
+        atomicAdd(st + kStMatched, static_cast<unsigned long long>(c_matched));
+        atomicAdd(st + kStTokensFullyReused, static_cast<unsigned long long>(c_full));
+        if (c_near) atomicAdd(st + kStNearScore, static_cast<unsigned long long>(c_near));
+      }
+      if (blockIdx.x == 0) {
+        const unsigned long long br = static_cast<unsigned long long>(sel.T) * k;
+        atomicAdd(st + kStLayerSteps, 1ull);
+        atomicAdd(st + kStBranches, br);
+        if (sel.refresh) atomicAdd(st + kStRefreshSteps, 1ull);
+        else atomicAdd(st + kStCacheBranches, br);
+      }
+    }
+  }
+
+  // Rows per group of the blocks before this one and of all blocks: a group's
+  // blocks in R ranges, one thread each, added in range order.
+  {
+    const int nb = gridDim.x, me = blockIdx.x;
+    const int R = kDecThreads / G, g = t % G, j = t / G;
+    int pre = 0, tot = 0;
+    bool ok = true;
+    if (j < R) {
+      const int lo = static_cast<int>(static_cast<long long>(j) * nb / R);
+      const int hi = static_cast<int>(static_cast<long long>(j + 1) * nb / R);
+      ok = read_tagged<16>(
+          a.words, hi - lo, [&](int q) { return static_cast<size_t>(lo + q) * G + g; }, epoch,
+          globaltimer() + kDecWaitNs, [&](int q, uint32_t v) {
+            const int c = static_cast<int>(v);
+            if (lo + q < me) pre += c;
+            tot += c;
+          });
+    }
+    if (!ok) {
+      report_status(sel.status, kStatusWaitTimeout, 620);
+      s_fail = 1;
+    }
+    s_part[t][0] = pre;
+    s_part[t][1] = tot;
+    __syncthreads();
+    if (s_fail) return;
+    for (int gg = t; gg < G; gg += kDecThreads) {
+      int p2 = 0, t2 = 0;
+      for (int jj = 0; jj < R; ++jj) {
+        p2 += s_part[jj * G + gg][0];
+        t2 += s_part[jj * G + gg][1];
+      }
+      s_pre[gg] = p2;
+      s_tot[gg] = t2;
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    // Exclusive scan of the group totals into offsets, 32 groups at a time.
+    int carry = 0;
+    for (int g0 = 0; g0 < G; g0 += 32) {
+      const int g = g0 + lane;
+      const int v = g < G ? s_tot[g] : 0;
+      int incl = v;
+#pragma unroll
+      for (int dd = 1; dd < 32; dd <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, dd);
+        if (lane >= dd) incl += u;
+      }
+      if (g < G) s_off[g] = carry + incl - v;
+      carry += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) s_off[G] = carry;
+    __syncwarp();
+    // The block's row lists, ascending tokens within each group.
+    const unsigned lt = (1u << lane) - 1u;
+    const int i = tok0 + lane;
+#pragma unroll
+    for (int p = 0; p < KMAX; ++p) {
+      int pos = -1;
+      if (d.rec[p]) {
+        const int g = d.e[p];
+        pos = s_off[g] + s_pre[g] + __popc(s_bal[g] & lt);
+        a.list[pos] = i * k + d.sl[p];
+      }
+      s_pos[lane][p] = pos;
+    }
+    int pos = -1;
+    if (d.shared_row) {
+      pos = s_off[E] + s_pre[E] + __popc(s_bal[E] & lt);
+      a.list[pos] = i;
+    }
+    s_pos[lane][KMAX] = pos;
+  }
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    if (t == 0) *a.epoch = epoch;
+    for (int g = t; g < G; g += kDecThreads) sel.counts[g] = s_tot[g];
+    for (int g = t; g <= G; g += kDecThreads) sel.offsets[g] = s_off[g];
+  }
+  if (!a.xg) return;
+  // One warp per token: its row, read once, to each of its places.
+  constexpr int kC = 4;
+  const uint4* x = static_cast<const uint4*>(a.x);
+  uint4* xg = static_cast<uint4*>(a.xg);
+  const int nv = a.row_vecs;
+  for (int q = warp; q < ntok; q += kDecThreads / 32) {
+    const uint4* src = x + static_cast<size_t>(tok0 + q) * nv;
+    for (int c0 = lane; c0 < nv; c0 += 32 * kC) {
+      uint4 v[kC];
+#pragma unroll
+      for (int u = 0; u < kC; ++u)
+        if (c0 + 32 * u < nv) v[u] = src[c0 + 32 * u];
+#pragma unroll
+      for (int p = 0; p <= KMAX; ++p) {
+        const int pos = s_pos[q][p];
+        if (pos < 0) continue;
+        uint4* dst = xg + static_cast<size_t>(pos) * nv;
+#pragma unroll
+        for (int u = 0; u < kC; ++u)
+          if (c0 + 32 * u < nv) dst[c0 + 32 * u] = v[u];
+      }
+    }
+  }
+}
+
+template <typename F>
+auto with_kmax(int k, F&& f) {
+  if (k <= 2) return f(decide_kernel<2>);
+  if (k <= 4) return f(decide_kernel<4>);
+  return f(decide_kernel<kMaxTopK>);
+}
+
 }  // namespace
+
+int decide_blocks(int max_tokens, int k, int n_sms) {
+  const int nb = (max_tokens + kDecTokens - 1) / kDecTokens;
+  int occ = 0;
+  const cudaError_t e = with_kmax(k, [&](auto kern) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kDecThreads, 0);
+  });
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return static_cast<long long>(occ) * n_sms >= nb ? nb : 0;
+}
+
+cudaError_t launch_decide(const DecideArgs& a, cudaStream_t s) {
+  const dim3 grid((a.sel.T + kDecTokens - 1) / kDecTokens);
+  return with_kmax(a.sel.k, [&](auto kern) { return launch_pdl(kern, grid, dim3(kDecThreads), 0, s, a); });
+}
 
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t s) {
   const int grid = (a.T + kThreads - 1) / kThreads;

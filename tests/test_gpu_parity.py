@@ -344,3 +344,72 @@ def test_single_layer_steps_back_to_back(M):
         st.close()
     for a, b in zip(*outs):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("D,E,k,S,bf16,cfg_kw", [
+    (128, 64, 8, 0, True, dict(ffn_impl=1)),   # widest groups and rows per token
+    (128, 7, 3, 1, True, dict(ffn_impl=1)),    # a shared expert, groups not dividing the block
+    (132, 8, 2, 0, False, {}),                 # fp32, a row of 33 16-byte vectors
+    (64, 1, 1, 0, False, {}),                  # a single expert
+    (256, 4, 4, 1, False, dict(shared_policy=1, reused_meta_policy=1)),
+])
+@pytest.mark.parametrize("T", [1, 33, 300])
+def test_decide_kernel_matches_the_three_kernels(M, D, E, k, S, bf16, cfg_kw, T):
+    """Selection, compaction and row gather in one launch (a handle of T
+    tokens) against the three kernels, which a handle of more tokens than can
+    be resident at once uses: the same bits everywhere."""
+    F, res = 64, []
+    for max_tokens in (T, 16000):  # 500 blocks; at most 3 of them fit an SM
+        w, x0, rng = W.tiny_layer(35, T, D, E, k, F, n_shared=S, dtype="bf16" if bf16 else "f32", bias=True,
+                                  wscale=0.05)
+        cfg = M.moeca_config_default(n_layers=1, hidden=D, ffn=F, n_experts=E, top_k=k, n_shared=S,
+                                     max_tokens=max_tokens, dtype=M.MOECA_BF16 if bf16 else M.MOECA_F32,
+                                     tau0=1.3 / k, **cfg_kw)
+        st = M.Stack(cfg, [w])
+        xs = drift(x0, rng, 4, 0.05, bf16)
+        got = []
+        for t, x in enumerate(xs):
+            got.append(st.step(torch.from_numpy(x).cuda().to(torch.bfloat16 if bf16 else torch.float32), t))
+            tr = st.get_trace(0, T)
+            n = int(tr["offsets"][-1])
+            got += [tr[f] for f in ("recompute", "slot", "matched", "token_any", "counts", "offsets")] + [tr["list"][:n]]
+        s = st.get_state(0)
+        got += [s[f] for f in ("cache_e", "cache_w", "cache_norm", "cache_h")]
+        res.append((got, st.stats()))
+        st.close()
+    assert res[0][1] == res[1][1]
+    for a, b in zip(res[0][0], res[1][0]):
+        assert torch.equal(a, b)
+
+
+def test_separate_path_step_replays_from_a_graph(M):
+    """A captured cache step of the separate path, replayed with new inputs in
+    the same buffer, gives the bits of steps launched one by one."""
+    T, D, E, k, F = 300, 128, 8, 2, 256
+    w, x0, rng = W.tiny_layer(36, T, D, E, k, F, wscale=0.05)
+    xs = [torch.from_numpy(x).cuda() for x in drift(x0, rng, 6, 0.05, False)]
+    cfg = M.moeca_config_default(n_layers=1, hidden=D, ffn=F, n_experts=E, top_k=k, max_tokens=T,
+                                 dtype=M.MOECA_F32, tau0=0.75)
+    ref = M.Stack(cfg, [w])
+    want = [ref.step(x, t).clone() for t, x in enumerate(xs)]
+    assert 0 < ref.stats()["reused"] < ref.stats()["cache_step_branches"]
+    ref.close()
+    st = M.Stack(cfg, [w])
+    x, out = xs[0].clone(), torch.empty_like(xs[0])
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        for t in (0, 1):
+            x.copy_(xs[t])
+            st.step(x, t, out=out)
+            assert torch.equal(out, want[t])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        st.step(x, 2, out=out)
+    for t in range(2, 6):
+        x.copy_(xs[t])
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want[t]), t
+    st.close()
