@@ -464,8 +464,8 @@ moeca_status moeca_destroy(moeca_handle* h);
  * The first call on each device looks up that device's address of the scratch
  * array (cudaGetSymbolAddress, with that device current), so make the first
  * call on a device before any stream capture.  Every call shares the one
- * array, which keeps the last call's contents; each call clears what must
- * start at zero itself.  Calls that overlap on the GPU (on different streams
+ * array, which keeps the last call's contents; what must start at zero is left
+ * at zero by the call before.  Calls that overlap on the GPU (on different streams
  * or from different host threads) race on the scratch: serialise them.
  * Runs on the current device, asynchronously on `stream`. */
 typedef struct {

@@ -557,12 +557,11 @@ extern "C" moeca_status moeca_route_noalloc(const moeca_route_args* r, void* str
     base = g_scratch_addr[dev];
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // The ticket and the counters must start at zero; the partials are written
-  // by every block before the last block reads them.
-  if (cudaMemsetAsync(base, 0, kScratchHeader, s) != cudaSuccess) {
-    cudaGetLastError();
-    return MOECA_ERR_CUDA;
-  }
+  // The ticket starts at zero (the array is zero when loaded, and the last
+  // block of every launch sets it back), the near-tie counter only counts, and
+  // the partials are written by every block before the last block reads them.
+  // Clearing the header with a memset before each launch cost 3.5 of 14.3 us a
+  // call (512 tokens, D 384, 8 experts, fp32).
   RouterArgs a{};
   a.x = r->x;
   a.w_gate = r->w_gate;
