@@ -8,6 +8,7 @@
 // (group, m-tile) from them; blocks past the last tile exit.  fp32 FFMA with
 // fp32 accumulation: the fp32 debug-precision path, and a cross-check of the
 // tensor-core kernel on bf16.
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -129,136 +130,144 @@ __device__ __forceinline__ void cp_async16_zf(uint32_t dst, const void* src, boo
 // PBM rows per tile (64 or 32), 4 PBM threads; thread (ty, tx) owns outputs
 // (ty + PBM/4 r, tx + 16 c).
 template <int PHASE, int PBM>
-__global__ void __launch_bounds__(4 * PBM) ffn_simt_pipe_kernel(FfnArgs a) {
+__global__ void __launch_bounds__(4 * PBM) ffn_simt_pipe_kernel(FfnArgs a, int S) {
   constexpr int NT = 4 * PBM, RS = PBM / 4;
   pdl_entry();
   const int N = PHASE == 1 ? a.F : a.D;
   const int K = PHASE == 1 ? a.D : a.F;
-  // The group sizes, loaded at once, then this block's (group, m-tile).
+  // The group sizes, loaded at once, then this block's tiles: unit u is n-tile
+  // u % ntiles of m-tile (u / ntiles) % m-tiles and K split u / (both).
   __shared__ int cnt_sm[kMaxExperts + 1];
   for (int gg = threadIdx.x; gg < a.G; gg += NT) cnt_sm[gg] = a.counts[gg];
   __syncthreads();
-  int mt = blockIdx.y, g = -1, m0 = 0;
-  for (int gg = 0; gg < a.G; ++gg) {
-    const int tiles = (cnt_sm[gg] + PBM - 1) / PBM;
-    if (mt < tiles) {
-      g = gg;
-      m0 = mt * PBM;
-      break;
+  int m_tiles = 0;
+  for (int gg = 0; gg < a.G; ++gg) m_tiles += (cnt_sm[gg] + PBM - 1) / PBM;
+  const int n_tiles = (N + PBN - 1) / PBN;
+  const unsigned units = static_cast<unsigned>(m_tiles) * n_tiles * S;  // within 32 bits: the host checked
+  for (unsigned unit = blockIdx.x; unit < units; unit += gridDim.x) {
+    const unsigned rest = unit / n_tiles;
+    const int nt = unit - rest * n_tiles, z = rest / m_tiles;
+    int mt = rest - static_cast<unsigned>(z) * m_tiles, g = 0, m0 = 0;
+    for (; g < a.G; ++g) {
+      const int tiles = (cnt_sm[g] + PBM - 1) / PBM;
+      if (mt < tiles) {
+        m0 = mt * PBM;
+        break;
+      }
+      mt -= tiles;
     }
-    mt -= tiles;
-  }
-  if (g < 0) return;
-  const int rows = cnt_sm[g];
-  const int row0 = a.offsets[g];
-  const int n0 = blockIdx.x * PBN;
-  const float* A = static_cast<const float*>(PHASE == 1 ? a.xg : a.hmid);
-  const float* B;
-  if (g < a.E) {
-    B = static_cast<const float*>(PHASE == 1 ? a.w1 : a.w2) + static_cast<size_t>(g) * a.F * a.D;
-  } else {
-    B = static_cast<const float*>(PHASE == 1 ? a.ws1 : a.ws2);
-  }
-  extern __shared__ __align__(16) float sm_pipe[];
-  float* As = sm_pipe;                    // [PST][PBM][PLD]
-  float* Bs = sm_pipe + PST * PBM * PLD;  // [PST][PBN][PLD]
-  const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
-  // K tiles of this block: all of them, or split z of blockIdx.z (second
-  // GEMM with K splits: whole tiles per split, partials written to a.partial).
-  const int KTA = (K + PBK - 1) / PBK, S = gridDim.z, z = blockIdx.z;
-  const int kt0 = z * KTA / S, KT = (z + 1) * KTA / S;
-  // Stage st <- K tile kt: rows x PBK / 4 chunks of 4 floats per operand (A:
-  // PBM rows, B: 64); chunks past K or past the rows are zeros.
-  constexpr int CPR = PBK / 4;
-  auto load = [&](int kt, int st) {
-    const int k0 = kt * PBK;
-#pragma unroll
-    for (int c = t; c < PBM * CPR; c += NT) {
-      const int r = c / CPR, kc = (c % CPR) * 4;
-      const bool va = k0 + kc < K && m0 + r < rows;
-      cp_async16_zf(smem_u32(As + (st * PBM + r) * PLD + kc),
-                    va ? A + static_cast<size_t>(row0 + m0 + r) * K + k0 + kc : A, va);
+    const int rows = cnt_sm[g];
+    const int row0 = a.offsets[g];
+    const int n0 = nt * PBN;
+    const float* A = static_cast<const float*>(PHASE == 1 ? a.xg : a.hmid);
+    const float* B;
+    if (g < a.E) {
+      B = static_cast<const float*>(PHASE == 1 ? a.w1 : a.w2) + static_cast<size_t>(g) * a.F * a.D;
+    } else {
+      B = static_cast<const float*>(PHASE == 1 ? a.ws1 : a.ws2);
     }
+    extern __shared__ __align__(16) float sm_pipe[];
+    float* As = sm_pipe;                    // [PST][PBM][PLD]
+    float* Bs = sm_pipe + PST * PBM * PLD;  // [PST][PBN][PLD]
+    const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
+    // K tiles of this unit: all of them, or split z of S (second GEMM with K
+    // splits: whole tiles per split, partials written to a.partial).
+    const int KTA = (K + PBK - 1) / PBK;
+    const int kt0 = z * KTA / S, KT = (z + 1) * KTA / S;
+    // Stage st <- K tile kt: rows x PBK / 4 chunks of 4 floats per operand (A:
+    // PBM rows, B: 64); chunks past K or past the rows are zeros.
+    constexpr int CPR = PBK / 4;
+    auto load = [&](int kt, int st) {
+      const int k0 = kt * PBK;
 #pragma unroll
-    for (int c = t; c < PBN * CPR; c += NT) {
-      const int r = c / CPR, kc = (c % CPR) * 4;
-      const bool vb = k0 + kc < K && n0 + r < N;
-      cp_async16_zf(smem_u32(Bs + (st * PBN + r) * PLD + kc),
-                    vb ? B + static_cast<size_t>(n0 + r) * K + k0 + kc : B, vb);
+      for (int c = t; c < PBM * CPR; c += NT) {
+        const int r = c / CPR, kc = (c % CPR) * 4;
+        const bool va = k0 + kc < K && m0 + r < rows;
+        cp_async16_zf(smem_u32(As + (st * PBM + r) * PLD + kc),
+                      va ? A + static_cast<size_t>(row0 + m0 + r) * K + k0 + kc : A, va);
+      }
+#pragma unroll
+      for (int c = t; c < PBN * CPR; c += NT) {
+        const int r = c / CPR, kc = (c % CPR) * 4;
+        const bool vb = k0 + kc < K && n0 + r < N;
+        cp_async16_zf(smem_u32(Bs + (st * PBN + r) * PLD + kc),
+                      vb ? B + static_cast<size_t>(n0 + r) * K + k0 + kc : B, vb);
+      }
+    };
+    float acc[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
+#pragma unroll
+    for (int st = 0; st < PST - 1; ++st) {
+      if (kt0 + st < KT) load(kt0 + st, st);
+      asm volatile("cp.async.commit_group;" ::: "memory");
     }
-  };
-  float acc[4][4];
+    for (int kt = kt0; kt < KT; ++kt) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(PST - 2) : "memory");
+      __syncthreads();  // tile kt is in; every thread is done with tile kt - 1
+      const int st = (kt - kt0) % PST;
+      const float* as = As + st * PBM * PLD;
+      const float* bs = Bs + st * PBN * PLD;
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+      for (int kk = 0; kk < PBK; kk += 4) {
+        float4 av[4], bv[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
+        for (int r = 0; r < 4; ++r) av[r] = *reinterpret_cast<const float4*>(as + (ty + RS * r) * PLD + kk);
 #pragma unroll
-  for (int st = 0; st < PST - 1; ++st) {
-    if (kt0 + st < KT) load(kt0 + st, st);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  }
-  for (int kt = kt0; kt < KT; ++kt) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(PST - 2) : "memory");
-    __syncthreads();  // tile kt is in; every thread is done with tile kt - 1
-    const int st = (kt - kt0) % PST;
-    const float* as = As + st * PBM * PLD;
-    const float* bs = Bs + st * PBN * PLD;
+        for (int c = 0; c < 4; ++c) bv[c] = *reinterpret_cast<const float4*>(bs + (tx + 16 * c) * PLD + kk);
 #pragma unroll
-    for (int kk = 0; kk < PBK; kk += 4) {
-      float4 av[4], bv[4];
+        for (int r = 0; r < 4; ++r)
 #pragma unroll
-      for (int r = 0; r < 4; ++r) av[r] = *reinterpret_cast<const float4*>(as + (ty + RS * r) * PLD + kk);
+          for (int c = 0; c < 4; ++c) {
+            acc[r][c] = fmaf(av[r].x, bv[c].x, acc[r][c]);
+            acc[r][c] = fmaf(av[r].y, bv[c].y, acc[r][c]);
+            acc[r][c] = fmaf(av[r].z, bv[c].z, acc[r][c]);
+            acc[r][c] = fmaf(av[r].w, bv[c].w, acc[r][c]);
+          }
+      }
+      // Refill the stage tile kt - 1 used.
+      const int nk = kt + PST - 1;
+      if (nk < KT) load(nk, (nk - kt0) % PST);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
 #pragma unroll
-      for (int c = 0; c < 4; ++c) bv[c] = *reinterpret_cast<const float4*>(bs + (tx + 16 * c) * PLD + kk);
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < 4; ++r) {
+      const int m = m0 + ty + RS * r;
+      if (m >= rows) continue;
+      const size_t row = static_cast<size_t>(row0 + m);
+      if (PHASE == 1) {
+        float* H = static_cast<float*>(a.hmid);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          acc[r][c] = fmaf(av[r].x, bv[c].x, acc[r][c]);
-          acc[r][c] = fmaf(av[r].y, bv[c].y, acc[r][c]);
-          acc[r][c] = fmaf(av[r].z, bv[c].z, acc[r][c]);
-          acc[r][c] = fmaf(av[r].w, bv[c].w, acc[r][c]);
+          const int n = n0 + tx + 16 * c;
+          if (n < N) H[row * a.F + n] = gelu_f(acc[r][c], a.gelu_tanh);
         }
-    }
-    // Refill the stage tile kt - 1 used.
-    const int nk = kt + PST - 1;
-    if (nk < KT) load(nk, (nk - kt0) % PST);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  }
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
+      } else if (S > 1) {
+        float* P = a.partial + (static_cast<size_t>(z) * a.max_rows + row) * a.D;
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int m = m0 + ty + RS * r;
-    if (m >= rows) continue;
-    const size_t row = static_cast<size_t>(row0 + m);
-    if (PHASE == 1) {
-      float* H = static_cast<float*>(a.hmid);
+        for (int c = 0; c < 4; ++c) {
+          const int n = n0 + tx + 16 * c;
+          if (n < N) P[n] = acc[r][c];
+        }
+      } else {
+        const int dr = a.list[row];
+        const int lim = g < a.E ? a.T * a.k : a.T;
+        if (dr < 0 || dr >= lim) {
+          report_status(a.status, kStatusBadIndex, 2000000 + static_cast<int>(row));
+          continue;
+        }
+        float* dst = static_cast<float*>(g < a.E ? a.cache_h : a.shared_h);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int n = n0 + tx + 16 * c;
-        if (n < N) H[row * a.F + n] = gelu_f(acc[r][c], a.gelu_tanh);
-      }
-    } else if (S > 1) {
-      float* P = a.partial + (static_cast<size_t>(z) * a.max_rows + row) * a.D;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int n = n0 + tx + 16 * c;
-        if (n < N) P[n] = acc[r][c];
-      }
-    } else {
-      const int dr = a.list[row];
-      const int lim = g < a.E ? a.T * a.k : a.T;
-      if (dr < 0 || dr >= lim) {
-        report_status(a.status, kStatusBadIndex, 2000000 + static_cast<int>(row));
-        continue;
-      }
-      float* dst = static_cast<float*>(g < a.E ? a.cache_h : a.shared_h);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int n = n0 + tx + 16 * c;
-        if (n < N) dst[static_cast<size_t>(dr) * a.D + n] = acc[r][c];
+        for (int c = 0; c < 4; ++c) {
+          const int n = n0 + tx + 16 * c;
+          if (n < N) dst[static_cast<size_t>(dr) * a.D + n] = acc[r][c];
+        }
       }
     }
+    __syncthreads();  // every thread is done with the stages before the next unit refills them
   }
 }
 
@@ -312,12 +321,14 @@ __global__ void __launch_bounds__(256) ffn_split_sum_kernel(FfnArgs a) {
 #define PIPE_BM2 32
 #endif
 
-// Plain launches: the grid covers the worst case, and its blocks launched
-// early under a programmatic dependency would sit resident beside the
-// previous kernel's blocks and slow them (measured: 455 vs 209 us per step
-// of the fp32 workload).
+// The pipelined kernels run a grid of at most the blocks that fit the GPU at
+// once, each striding over the launch's tiles, so that they can be launched
+// early under the programmatic dependency: a grid of the worst case's blocks
+// sat beside the previous kernel's and slowed them (fp32 workload: 455 vs
+// 209 us per step), and plain launches left the gaps between the kernels open
+// (4 steps, D 384, 512 tokens: 368 us, now 358).  The plain form keeps the worst case's grid and plain launches.
 template <typename TI>
-cudaError_t launch_t(const FfnArgs& a, int phase, cudaStream_t s) {
+cudaError_t launch_t(const FfnArgs& a, int phase, int n_sms, cudaStream_t s) {
   const int N = phase == 1 ? a.F : a.D;
   auto al16 = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
   if (std::is_same_v<TI, float> && a.D % 4 == 0 && a.F % 4 == 0 && al16(a.xg) && al16(a.hmid) && al16(a.w1) &&
@@ -326,9 +337,14 @@ cudaError_t launch_t(const FfnArgs& a, int phase, cudaStream_t s) {
     auto run = [&](auto kern, int bm, size_t smem, int splits) -> cudaError_t {
       const cudaError_t e = set_dyn_smem_on_device(reinterpret_cast<const void*>(kern), static_cast<int>(smem));
       if (e != cudaSuccess) return e;
-      const dim3 grid((N + PBN - 1) / PBN, (a.max_rows + bm - 1) / bm + a.G, splits);
-      kern<<<grid, 4 * bm, smem, s>>>(a);
-      return cudaGetLastError();
+      const long long units =
+          static_cast<long long>((N + PBN - 1) / PBN) * ((a.max_rows + bm - 1) / bm + a.G) * splits;
+      if (units > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+      int occ = 0;
+      const cudaError_t oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 4 * bm, smem);
+      if (oe != cudaSuccess) return oe;
+      const dim3 grid(static_cast<unsigned>(std::min<long long>(units, static_cast<long long>(std::max(occ, 1)) * n_sms)));
+      return launch_pdl(kern, grid, dim3(4 * bm), smem, s, a, splits);
     };
     if (phase == 1) return run(ffn_simt_pipe_kernel<1, PIPE_BM1>, PIPE_BM1, pipe_smem<PIPE_BM1>(), 1);
     // The second GEMM has few outputs and a long K: K splits give the SMs
@@ -336,8 +352,7 @@ cudaError_t launch_t(const FfnArgs& a, int phase, cudaStream_t s) {
     const int splits = a.partial && a.simt_split > 1 && a.D % 4 == 0 ? a.simt_split : 1;
     const cudaError_t e = run(ffn_simt_pipe_kernel<2, PIPE_BM2>, PIPE_BM2, pipe_smem<PIPE_BM2>(), splits);
     if (e != cudaSuccess || splits == 1) return e;
-    ffn_split_sum_kernel<<<(a.max_rows + 7) / 8, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(ffn_split_sum_kernel, dim3(std::min((a.max_rows + 7) / 8, 8 * n_sms)), dim3(256), 0, s, a);
   }
   const dim3 grid((N + BN - 1) / BN, (a.max_rows + BM - 1) / BM + a.G);
   if (phase == 1) ffn_simt_kernel<TI, 1><<<grid, 256, 0, s>>>(a);
@@ -347,8 +362,8 @@ cudaError_t launch_t(const FfnArgs& a, int phase, cudaStream_t s) {
 
 }  // namespace
 
-cudaError_t launch_ffn_simt(const FfnArgs& a, bool bf16, int phase, cudaStream_t s) {
-  return bf16 ? launch_t<__nv_bfloat16>(a, phase, s) : launch_t<float>(a, phase, s);
+cudaError_t launch_ffn_simt(const FfnArgs& a, bool bf16, int phase, int n_sms, cudaStream_t s) {
+  return bf16 ? launch_t<__nv_bfloat16>(a, phase, n_sms, s) : launch_t<float>(a, phase, n_sms, s);
 }
 
 }  // namespace moeca

@@ -140,7 +140,7 @@ struct FfnArgs {
                          // kernel that follows re-arms it)
   int* status;
 };
-cudaError_t launch_ffn_simt(const FfnArgs& a, bool bf16, int phase, cudaStream_t s);
+cudaError_t launch_ffn_simt(const FfnArgs& a, bool bf16, int phase, int n_sms, cudaStream_t s);
 
 // tcgen05 / TMA grouped GEMM (bf16 only).  Tensor maps are built once per
 // handle; `TcPlan` owns them.

@@ -869,7 +869,7 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
     } else {
       for (int phase = 1; phase <= 2 && e == cudaSuccess; ++phase) {
         const int kind = phase == 1 ? MOECA_K_FFN1 : MOECA_K_FFN2;
-        e = timed(h, kind, s, [&] { return launch_ffn_simt(fa, h->bf16, phase, s); });
+        e = timed(h, kind, s, [&] { return launch_ffn_simt(fa, h->bf16, phase, h->n_sms, s); });
       }
     }
     if (e != cudaSuccess) break;
