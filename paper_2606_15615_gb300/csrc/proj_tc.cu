@@ -61,8 +61,10 @@ constexpr int kSub = 2;                 // K sub-blocks per stage
 constexpr int kMaxN = 256;              // token rows per tile
 constexpr int kBoxes = kMaxN / 32;      // token boxes of 16, 32, .., 128 rows
 constexpr int kMaxStages = 5;
-constexpr int kRingBytes = 208 * 1024;
+constexpr int kRingBytes = 208 * 1024;   // weight slots first, then token slots
+constexpr int kEarly = 3;                // stages (every ring has as many) whose weights load before the wait
 constexpr int kABytes = kBM * kBK * 2;  // 16 KB: one weight sub-block
+constexpr int kWSlot = kSub * kABytes;  // a stage's weights
 constexpr int kEpiWarps = 8;            // warps 2-9
 constexpr int kTokWarp = 2 + kEpiWarps;
 constexpr int kPThreads = 32 * (kTokWarp + 1);
@@ -192,17 +194,28 @@ __global__ void __launch_bounds__(kPThreads, 1)
   cluster_arrive();
   cluster_wait();  // both CTAs' barriers are initialised, TMEM is allocated
   tc_fence_after();
+  const uint32_t ring = smem_u32(smem);
+  const int nw = (p.N + 2 * kBM - 1) / (2 * kBM);
+  const int sub = p.K / kBK, ks = (sub + kSub - 1) / kSub;
+  // The weights of the first tile's first stages load before the dependency
+  // wait: which they are does not depend on the row count.  Their bytes
+  // complete on the stages' barriers, which the leader arms after the wait.
+  const int early = min(kEarly, ks), w_first = pair % nw;
+  if (warp == 0 && lane == 0) {
+    const int feat = w_first * 2 * kBM + static_cast<int>(rank) * kBM;
+    const uint32_t full0 = cluster_addr(smem_u32(&full_bar[0]), 0);
+    for (int k = 0; k < early && feat < p.N; ++k)
+      tma_load_k64_pair(ring + k * kWSlot, &maps.w, feat, k * kSub, full0 + k * 8);
+  }
   pdl_entry();
   const int M = p.m_dev ? min(*reinterpret_cast<const volatile int*>(p.m_dev), p.M) : p.M;
   if (p.row_stat && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(p.row_stat, static_cast<unsigned long long>(M));
   const uint32_t tmem = tmem_sh;
-  const int nw = (p.N + 2 * kBM - 1) / (2 * kBM);
   const int n = token_width(M, nw, n_pairs), half = n >> 1;
   const int units = (M + n - 1) / n * nw;
-  const int sub = p.K / kBK, ks = (sub + kSub - 1) / kSub;
-  const int slot_bytes = kSub * (kABytes + half * (kBK * 2));
-  const int nst = min(kMaxStages, kRingBytes / slot_bytes);
-  const uint32_t ring = smem_u32(smem), ring_end = ring + nst * slot_bytes;
+  const int t_slot = kSub * half * (kBK * 2);  // a stage's token rows
+  const int nst = min(kMaxStages, kRingBytes / (kWSlot + t_slot));
+  const uint32_t ring_t = ring + nst * kWSlot;
   const uint32_t empty0 = smem_u32(&empty_bar[0]);
 
   if (warp == 0 || warp == kTokWarp) {
@@ -210,7 +223,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
       // ---------------- TMA producers: weights (warp 0), tokens ----------------
       const bool wts = warp == 0;
       const CUtensorMap* map = wts ? &maps.w : &maps.act[(n >> 5) - 1];
-      const uint32_t first = ring + (wts ? 0 : kSub * kABytes), end = first + nst * slot_bytes;
+      const int slot_bytes = wts ? kWSlot : t_slot;
+      const uint32_t first = wts ? ring : ring_t, end = first + nst * slot_bytes;
       const uint32_t full0 = cluster_addr(smem_u32(&full_bar[0]), 0);
       uint32_t dst = first, eb = empty0, fb = full0, par = 1u;
       int issued = 0;
@@ -227,7 +241,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
           // the leader arms its barrier with the bytes of both CTAs.
           if (!(ok = mbar_wait_hot(eb, par, &abort_flag))) break;
           if (wts && rank == 0) mbar_expect_tx(fb, tx);
-          if (live) tma_load_k64_pair(dst, map, row, k * kSub, fb);
+          if (live && !(wts && issued < early)) tma_load_k64_pair(dst, map, row, k * kSub, fb);
           ++issued;
           dst += slot_bytes;
           eb += 8;
@@ -239,6 +253,12 @@ __global__ void __launch_bounds__(kPThreads, 1)
             par ^= 1u;
           }
         }
+      }
+      if (wts && rank == 0 && pair >= units) {
+        // No tile for this pair: the early copies land before the CTAs exit.
+        const uint32_t tx = kWSlot * (w_first * 2 * kBM + kBM < p.N ? 2 : 1);
+        for (int k = 0; k < early; ++k) mbar_expect_tx(smem_u32(&full_bar[k]), tx);
+        for (int k = 0; k < early && ok; ++k) ok = mbar_wait(smem_u32(&full_bar[k]), 0, &abort_flag);
       }
       if (!ok) {
         if (!abort_flag) report_status(p.status, kStatusWaitTimeout, wts ? 600 : 603);
@@ -256,11 +276,11 @@ __global__ void __launch_bounds__(kPThreads, 1)
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
       // ---------------- MMA issuer (the leader, for both CTAs) ----------------
-      const uint32_t w_lo0 = ((ring & 0x3FFFFu) >> 4) | (1u << 16), slot_lo = static_cast<uint32_t>(slot_bytes) >> 4;
-      const uint32_t w_end = ((ring_end & 0x3FFFFu) >> 4) | (1u << 16);
+      const uint32_t w_lo0 = ((ring & 0x3FFFFu) >> 4) | (1u << 16), x_lo0 = ((ring_t & 0x3FFFFu) >> 4) | (1u << 16);
       const uint32_t full0 = smem_u32(&full_bar[0]);
       const uint32_t idesc = instr_desc(2 * kBM, n), b_sub = n * kBK >> 4;
-      uint32_t w_lo = w_lo0, fb = full0, eb = empty0, par = 0u, acc_phase = 0;
+      const uint32_t x_end = x_lo0 + nst * (static_cast<uint32_t>(t_slot) >> 4);
+      uint32_t w_lo = w_lo0, x_lo = x_lo0, fb = full0, eb = empty0, par = 0u, acc_phase = 0;
       int acc = 0;
       bool ok = true;
       for (int u = pair; u < units; u += n_pairs) {
@@ -273,17 +293,19 @@ __global__ void __launch_bounds__(kPThreads, 1)
 #pragma unroll
           for (int q = 0; q < kSub; ++q) {
             if (q && k * kSub + q >= sub) break;
-            const uint32_t wq = w_lo + q * (kABytes >> 4), xq = w_lo + (kSub * kABytes >> 4) + q * b_sub;
+            const uint32_t wq = w_lo + q * (kABytes >> 4), xq = x_lo + q * b_sub;
 #pragma unroll
             for (int kk = 0; kk < kBK / 16; ++kk)
               mma_bf16_pair(d_tmem, wq + kk * 2, xq + kk * 2, idesc, k != 0 || q != 0 || kk != 0);
           }
           mma_commit_pair(eb);
-          w_lo += slot_lo;
+          w_lo += kWSlot >> 4;
+          x_lo += static_cast<uint32_t>(t_slot) >> 4;
           fb += 8;
           eb += 8;
-          if (w_lo == w_end) {
+          if (x_lo == x_end) {
             w_lo = w_lo0;
+            x_lo = x_lo0;
             fb = full0;
             eb = empty0;
             par ^= 1u;
