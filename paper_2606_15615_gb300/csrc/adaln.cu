@@ -148,11 +148,12 @@ __device__ __forceinline__ void row_stats(const uint4* v, int nvec, int lane, in
   rstd = rsqrtf(warp_sum(ss) / static_cast<float>(D) + eps);
 }
 
-// dst = bf16((v - mean) rstd (1 + scale) + shift), chunk by chunk.
+// dst = bf16((v - mean) rstd (1 + scale) + shift), chunk by chunk; also to
+// dst2 and to the rows row_of[0 .. row_w) of xg that are not -1.
 template <int C>
 __device__ __forceinline__ void store_modulated(const uint4* v, int nvec, int lane, float mean, float rstd,
                                                 const float* shift, const float* scale, __nv_bfloat16* dst,
-                                                __nv_bfloat16* dst2) {
+                                                __nv_bfloat16* dst2, const int32_t* row_of, int row_w, uint4* xg) {
 #pragma unroll
   for (int q = 0; q < C; ++q) {
     const int c = lane + 32 * q;
@@ -166,6 +167,10 @@ __device__ __forceinline__ void store_modulated(const uint4* v, int nvec, int la
       const uint4 o = pack8(f);
       reinterpret_cast<uint4*>(dst)[c] = o;
       if (dst2) reinterpret_cast<uint4*>(dst2)[c] = o;
+      for (int r = 0; r < row_w; ++r) {
+        const int pos = __ldg(row_of + r);
+        if (pos >= 0) xg[static_cast<size_t>(pos) * nvec + c] = o;
+      }
     }
   }
 }
@@ -227,7 +232,8 @@ __global__ void __launch_bounds__(kLnWarps * 32) adaln_rows_kernel(AdaLnArgs a) 
   float mean, rstd;
   if (a.h_out) {
     row_stats<C>(v, nvec, lane, D, a.eps, mean, rstd);
-    store_modulated<C>(v, nvec, lane, mean, rstd, md, md + D, static_cast<__nv_bfloat16*>(a.h_out) + off, nullptr);
+    store_modulated<C>(v, nvec, lane, mean, rstd, md, md + D, static_cast<__nv_bfloat16*>(a.h_out) + off, nullptr, nullptr,
+                       0, nullptr);
   }
   if (a4) {
     // u = bf16(x + gate_a a): one rounding of the fused product-sum.
@@ -254,7 +260,9 @@ __global__ void __launch_bounds__(kLnWarps * 32) adaln_rows_kernel(AdaLnArgs a) 
     row_stats<C>(v, nvec, lane, D, a.eps, mean, rstd);
     store_modulated<C>(v, nvec, lane, mean, rstd, md + 3 * D, md + 4 * D,
                     static_cast<__nv_bfloat16*>(a.m_out) + off,
-                    a.m_copy ? static_cast<__nv_bfloat16*>(a.m_copy) + off : nullptr);
+                    a.m_copy ? static_cast<__nv_bfloat16*>(a.m_copy) + off : nullptr,
+                    a.row_of ? a.row_of + static_cast<size_t>(t) * a.row_w : nullptr, a.row_of ? a.row_w : 0,
+                    static_cast<uint4*>(a.xg));
   }
 }
 

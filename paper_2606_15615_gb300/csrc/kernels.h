@@ -204,10 +204,12 @@ struct PrepShape {
   bool attn;              // the DiT-MoE block build of the kernel
 };
 constexpr size_t kPrepSmemMax = 200 * 1024;
-PrepShape prep_plan(int D, int E, int k, int max_tokens, int n_sms, bool attn);
+// attn: the DiT-MoE block build; stage_a: its blocks also stage the cached
+// attention rows (a block without AdaLN, whose router input is x + a^{t0}).
+PrepShape prep_plan(int D, int E, int k, int max_tokens, int n_sms, bool attn, bool stage_a);
 // The two builds of prep.cu (plain, and prep_attn.cu for DiT-MoE blocks).
 PrepShape prep_plan_plain(int D, int E, int k, int max_tokens, int n_sms);
-PrepShape prep_plan_attn(int D, int E, int k, int max_tokens, int n_sms);
+PrepShape prep_plan_attn(int D, int E, int k, int max_tokens, int n_sms, bool stage_a);
 cudaError_t launch_prep_plain(const PrepArgs& a, const PrepShape& p, cudaStream_t s);
 cudaError_t launch_prep_attn(const PrepArgs& a, const PrepShape& p, cudaStream_t s);
 cudaError_t launch_prep(const PrepArgs& a, const PrepShape& p, cudaStream_t s);
@@ -307,6 +309,9 @@ struct AdaLnArgs {
   void* m_copy;           // [T, D] or null
   const int32_t* rows;    // or null (every row)
   const int* n_rows;      // device count of rows (with rows)
+  const int32_t* row_of;  // with rows, or null: [T, row_w] FFN row positions of the token (-1: none);
+  int row_w;              //   m is also written to those rows of xg
+  void* xg;               // [rows, D] FFN input rows
   int* status;
 };
 constexpr int kAdaLnMaxD = 2560;

@@ -581,9 +581,8 @@ moeca_status moeca_create(const moeca_config* cfg, const moeca_layer_weights* la
     h->tc_dep_pairs_n = static_cast<int>(tc_dep_pairs(h->max_rows, h->G));
     A((void**)&h->tc_dep, static_cast<size_t>(h->tc_dep_pairs_n) * 2 * sizeof(int));
     A((void**)&h->tc_work, 2 * sizeof(int));
-    // An AdaLN block forms its router input in its own kernel: the plain
-    // preparation kernel, with the attention list built separately.
-    h->prep = prep_plan(c.hidden, c.n_experts, c.top_k, c.max_tokens, h->n_sms, attn && !ada);
+    // An AdaLN block forms its router input in its own kernel.
+    h->prep = prep_plan(c.hidden, c.n_experts, c.top_k, c.max_tokens, h->n_sms, attn, attn && !ada);
     if (h->prep.tokens_per_block) {
       const size_t nb = (T + h->prep.tokens_per_block - 1) / h->prep.tokens_per_block;
       h->prep_count_off = nb * E * 2;
@@ -797,21 +796,24 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
         pa.attn_a = L.attn_a;
         pa.u_out = L.attn_u;
       }
-      if (attn_sync && !ada) {
+      if (attn_sync) {
         // The recomputing-token list comes out of the same compaction.
         pa.attn_list = 1;
         pa.attn_rows = h->attn_rows; pa.attn_n = h->attn_n; pa.attn_inv = h->attn_inv;
         pa.sample_lo = h->attn_samp; pa.seq = seq;
       }
-      if (attn_sync && !ada) {
+      if (attn_sync) {
         // The rows of tokens that keep their attention are final now; the
-        // output projection writes the others (row_of says where).
+        // output projection (AdaLN: the row pass after it) writes the others
+        // (row_of says where).
         pa.xg = h->xg;
         pa.gather_final_only = 1;
         pa.row_of = h->attn_rowof;
-        oa.row_of = h->attn_rowof;
-        oa.row_w = c.top_k + c.n_shared;
-        oa.xg = h->xg;
+        if (!ada) {
+          oa.row_of = h->attn_rowof;
+          oa.row_w = c.top_k + c.n_shared;
+          oa.xg = h->xg;
+        }
       }
       if (++h->prep_epoch == 0) h->prep_epoch = 1;  // 0 marks words never written
       pa.epoch = pa.wait_epoch = h->prep_epoch;
@@ -837,7 +839,7 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
       // Sec. 4.1: the tokens with a non-empty recompute set recompute their
       // attention output over all keys of their sample; their a and u rows
       // are replaced, then the FFN rows are gathered from u.
-      if ((!fused || ada) && (e = timed(h, MOECA_K_ATTN_AUX, s, [&] {
+      if (!fused && (e = timed(h, MOECA_K_ATTN_AUX, s, [&] {
                        return launch_attn_rows(L.token_any, T, seq, h->attn_rows, h->attn_n, h->attn_samp,
                                                h->attn_inv, s);
                      })) != cudaSuccess)
@@ -851,9 +853,12 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
         // The listed tokens' MoE input m from their new u.
         AdaLnArgs mm = la;
         mm.m_out = L.attn_m; mm.rows = h->attn_rows; mm.n_rows = h->attn_n;
+        if (fused) {
+          mm.row_of = h->attn_rowof; mm.row_w = c.top_k + c.n_shared; mm.xg = h->xg;
+        }
         if ((e = timed(h, MOECA_K_ADALN, s, [&] { return launch_adaln_rows(mm, s); })) != cudaSuccess) break;
       }
-      if (!fused || ada) {
+      if (!fused) {
         CompactArgs ga = ca;
         ga.xg = h->xg;
         if ((e = timed(h, MOECA_K_ATTN_AUX, s, [&] { return launch_gather(ga, h->bf16, s); })) != cudaSuccess)

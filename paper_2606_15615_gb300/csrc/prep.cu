@@ -724,10 +724,10 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(PrepArgs a) {
 }
 
 template <int TB, int EPAD>
-size_t prep_smem(int D, bool attn) {
+size_t prep_smem(int D, bool stage_a) {
   const size_t ldw = static_cast<size_t>(D) + 8;
   const size_t rows = (EPAD + TB) * ldw * 2;                        // gate rows, token rows
-  const size_t a_rows = attn ? TB * ldw * 2 : 0;                    // cached attention rows
+  const size_t a_rows = stage_a ? TB * ldw * 2 : 0;                 // cached attention rows
   return rows + prep_region_bytes(TB, EPAD) + a_rows;
 }
 
@@ -803,11 +803,11 @@ cudaError_t launch_prep_shard(const PrepArgs& a, const PrepShape& p, int mode, c
 }
 #else
 #if MOECA_PREP_ATTN
-PrepShape prep_plan_attn(int D, int E, int k, int max_tokens, int n_sms) {
+PrepShape prep_plan_attn(int D, int E, int k, int max_tokens, int n_sms, bool stage_a) {
   const bool attn = true;
 #else
 PrepShape prep_plan_plain(int D, int E, int k, int max_tokens, int n_sms) {
-  const bool attn = false;
+  const bool attn = false, stage_a = false;
 #endif
   PrepShape p{0, 0, 0, 0};
   if (D % 16 || E < 1 || E > kMaxExperts || k < 1 || k > kMaxTopK) return p;
@@ -818,7 +818,7 @@ PrepShape prep_plan_plain(int D, int E, int k, int max_tokens, int n_sms) {
     const int nb = (max_tokens + TB - 1) / TB;
     const size_t smem = with_shape(TB, epad, km, [&]<int tb, int ep, int kk>() -> size_t {
       if constexpr (tb == 0) return 0;
-      else return prep_smem<tb, ep>(D, attn);
+      else return prep_smem<tb, ep>(D, stage_a);
     });
     if (smem == 0 || smem > kPrepSmemMax) continue;
     const int occ = with_shape(TB, epad, km, [&]<int tb, int ep, int kk>() -> int {
@@ -849,8 +849,8 @@ cudaError_t launch_prep_plain(const PrepArgs& a, const PrepShape& p, cudaStream_
 }
 
 #if !MOECA_PREP_ATTN
-PrepShape prep_plan(int D, int E, int k, int max_tokens, int n_sms, bool attn) {
-  return attn ? prep_plan_attn(D, E, k, max_tokens, n_sms) : prep_plan_plain(D, E, k, max_tokens, n_sms);
+PrepShape prep_plan(int D, int E, int k, int max_tokens, int n_sms, bool attn, bool stage_a) {
+  return attn ? prep_plan_attn(D, E, k, max_tokens, n_sms, stage_a) : prep_plan_plain(D, E, k, max_tokens, n_sms);
 }
 
 cudaError_t launch_prep(const PrepArgs& a, const PrepShape& p, cudaStream_t s) {
