@@ -78,48 +78,64 @@ __host__ __device__ constexpr size_t prep_region_bytes(int TB, int EPAD) {
   return (static_cast<size_t>(prep_wpg(TB)) * TB * (EPAD + 1) * 4 + 15) / 16 * 16;
 }
 
-// DiT-MoE block work kept out of line, so the MoE-only path's code (phases
-// run once per launch, on the critical path) is what it is without it.
-// Bulk copies of the block's cached attention rows a^{t0} (thread 0).
-static __device__ __noinline__ void issue_attn_rows(const PrepArgs& a, __nv_bfloat16* s_a, int ldw, int tok0,
-                                                    int ntok, uint32_t row_bytes, uint32_t bar) {
+// DiT-MoE block work, in that build only.
+// Bulk copies of the block's cached attention rows a^{t0}, one per lane of warp 0.
+__device__ __forceinline__ void issue_attn_rows(const PrepArgs& a, __nv_bfloat16* s_a, int ldw, int tok0, int ntok,
+                                                uint32_t row_bytes, uint32_t bar, int lane) {
   const __nv_bfloat16* ar = static_cast<const __nv_bfloat16*>(a.attn_a);
-  for (int q = 0; q < ntok; ++q)
+  for (int q = lane; q < ntok; q += 32)
     bulk_g2s(smem_u32(s_a + q * ldw), ar + static_cast<size_t>(tok0 + q) * a.D, row_bytes, bar);
 }
 
-// u = x + a^{t0} (rounded to bf16) in place of the staged x rows, and to u_out.
-static __device__ __noinline__ void form_u(const PrepArgs& a, __nv_bfloat16* s_x, const __nv_bfloat16* s_a, int ldw,
-                                           int tok0, int ntok, int t) {
+// u = x + a^{t0} (rounded to bf16) in place of the staged x rows, and to
+// u_out: one warp per row, four vectors of a lane in flight.
+__device__ __forceinline__ void form_u(const PrepArgs& a, __nv_bfloat16* s_x, const __nv_bfloat16* s_a, int ldw,
+                                       int tok0, int ntok, int t) {
   __nv_bfloat16* u_out = static_cast<__nv_bfloat16*>(a.u_out);
   const int nv = a.D / 8;
-  for (int idx = t; idx < ntok * nv; idx += kThreads) {
-    const int q = idx / nv, c = idx % nv;
-    uint4* xs = reinterpret_cast<uint4*>(s_x + q * ldw) + c;
-    float xv[8], av[8];
-    unpack_vec(*xs, xv, static_cast<__nv_bfloat16*>(nullptr));
-    unpack_vec(*(reinterpret_cast<const uint4*>(s_a + q * ldw) + c), av, static_cast<__nv_bfloat16*>(nullptr));
+  for (int q = t >> 5; q < ntok; q += kThreads / 32) {
+    uint4* xs = reinterpret_cast<uint4*>(s_x + q * ldw);
+    const uint4* as = reinterpret_cast<const uint4*>(s_a + q * ldw);
+    uint4* us = reinterpret_cast<uint4*>(u_out + static_cast<size_t>(tok0 + q) * a.D);
+    for (int c0 = t & 31; c0 < nv; c0 += 128) {
+      uint4 x[4], av[4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) xv[j] += av[j];
-    uint4 uv;
-    __nv_bfloat162* uh = reinterpret_cast<__nv_bfloat162*>(&uv);
+      for (int r = 0; r < 4; ++r)
+        if (c0 + 32 * r < nv) {
+          x[r] = xs[c0 + 32 * r];
+          av[r] = as[c0 + 32 * r];
+        }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) uh[j] = __floats2bfloat162_rn(xv[2 * j], xv[2 * j + 1]);
-    *xs = uv;
-    reinterpret_cast<uint4*>(u_out + static_cast<size_t>(tok0 + q) * a.D)[c] = uv;
+      for (int r = 0; r < 4; ++r)
+        if (c0 + 32 * r < nv) {
+          float xf[8], af[8];
+          unpack_vec(x[r], xf, static_cast<__nv_bfloat16*>(nullptr));
+          unpack_vec(av[r], af, static_cast<__nv_bfloat16*>(nullptr));
+          uint4 uv;
+          __nv_bfloat162* uh = reinterpret_cast<__nv_bfloat162*>(&uv);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            uh[j] = __floats2bfloat162_rn(xf[2 * j] + af[2 * j], xf[2 * j + 1] + af[2 * j + 1]);
+          xs[c0 + 32 * r] = uv;
+          us[c0 + 32 * r] = uv;
+        }
+    }
   }
 }
 
 // One lane's token (warp 0 of phase C): its FFN-row map entries (the list
 // positions of its recomputed branches, -1 elsewhere) and its place in the
 // recomputing-token list.  `pos[p]` are the positions the list loop wrote.
-static __device__ __noinline__ void attn_bookkeeping(const PrepArgs& a, int i, int lane, int ntok, bool any,
-                                                     const int* pos, int shared_pos, int list_pos) {
+template <int KMAX>
+__device__ __forceinline__ void attn_bookkeeping(const PrepArgs& a, int i, int lane, int ntok, bool any,
+                                                 const int (&pos)[KMAX], int shared_pos, int list_pos) {
   if (lane >= ntok) return;  // 16-token blocks: lanes 16-31 hold the next block's tokens
   if (a.row_of) {
     const int W = a.sel.k + a.n_shared;
     int32_t* row_of = a.row_of + static_cast<size_t>(i) * W;
-    for (int p = 0; p < a.sel.k; ++p) row_of[p] = pos[p];
+#pragma unroll
+    for (int p = 0; p < KMAX; ++p)
+      if (p < a.sel.k) row_of[p] = pos[p];
     if (a.n_shared) row_of[a.sel.k] = shared_pos;
   }
   if (a.attn_list) {
@@ -214,7 +230,7 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(PrepArgs a) {
     if (kRoute)
       for (int e = lane; e < E; e += 32) bulk_g2s(smem_u32(s_w + e * ldw), wg + static_cast<size_t>(e) * D, row_bytes, bar);
     if constexpr (kAttn) {
-      if (add_a && lane == 0) issue_attn_rows(a, s_a, ldw, tok0, ntok, row_bytes, bar);  // written on an earlier step
+      if (add_a) issue_attn_rows(a, s_a, ldw, tok0, ntok, row_bytes, bar, lane);  // written on an earlier step
     }
   }
   // Prefetch what later phases read: cached metadata and EMA rows.
