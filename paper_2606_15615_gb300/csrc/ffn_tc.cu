@@ -477,11 +477,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int ks = t.p ? p1.ks : p0.ks, S = t.p ? p1.S : p0.S, N = a.N[t.p];
         const CUtensorMap* tw = t.g < a.E ? &mp.w : &mp.ws;
         const int feat = t.w * 256 + static_cast<int>(rank) * kBM;
-        const bool live = feat < N;                 // this CTA's half of the weight tile has rows
-        const int wrow = (t.g < a.E ? t.g * N : 0) + feat;
+        // A half tile without weight rows is copied from past the map's last row
+        // (zeros, no traffic): a CTA that brought nothing could be lapped by the
+        // MMAs, and a barrier two phases on looks like one not yet completed.
+        const int wrow = feat < N ? (t.g < a.E ? t.g * N : 0) + feat : (t.g < a.E ? a.E * N : N);
         const int k0 = t.sp * ks / S, k1 = (t.sp + 1) * ks / S;  // stages of this unit
         // Bytes a stage brings into both CTAs (sub-blocks past the last are zero-filled).
-        const uint32_t stage_tx = kSub * (kABytes * (t.w * 256 + kBM < N ? 2 : 1) + t.n * (kBK * 2));
+        const uint32_t stage_tx = kSub * (2 * kABytes + t.n * (kBK * 2));
         int ticket = 0;
         int k = k0;
         for (int part = 0; part < 3 && ok; ++part) {
@@ -492,7 +494,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // done; the leader arms its barrier with the bytes of both CTAs.
             if (!(ok = mbar_wait_hot(eb, par, &abort_flag))) break;
             if (leader) mbar_expect_tx(fb, stage_tx);
-            if (live) tma_load_k64_pair(dst, tw, wrow, k * kSub, fb);
+            tma_load_k64_pair(dst, tw, wrow, k * kSub, fb);
             ++issued;
             dst += slot_bytes;
             eb += 8;
@@ -651,7 +653,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         abort_flag = 1;
       }
       // Every MMA this thread issued has completed once the drain barrier fires.
-      mma_commit_pair(smem_u32(&drain_bar));
+      mma_commit_pair(smem_u32(&drain_bar), 1);
       const unsigned long long t0 = globaltimer();
       while (!mbar_try(smem_u32(&drain_bar), 0) && globaltimer() - t0 < kWaitNs) {
       }

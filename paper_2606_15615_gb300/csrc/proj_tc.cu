@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
   if (warp == 0 && lane == 0) {
     const int feat = w_first * 2 * kBM + static_cast<int>(rank) * kBM;
     const uint32_t full0 = cluster_addr(smem_u32(&full_bar[0]), 0);
-    for (int k = 0; k < early && feat < p.N; ++k)
+    for (int k = 0; k < early; ++k)
       tma_load_k64_pair(ring + k * kWSlot, &maps.w, feat, k * kSub, full0 + k * 8);
   }
   pdl_entry();
@@ -233,15 +233,17 @@ __global__ void __launch_bounds__(kPThreads, 1)
         const int tt = u / nw, w = u - tt * nw;
         const int feat = w * 2 * kBM + static_cast<int>(rank) * kBM;
         const int row = wts ? feat : tt * n + static_cast<int>(rank) * half;
-        const bool live = !wts || feat < p.N;  // this CTA's half of the weight tile has rows
-        // Bytes a stage brings into both CTAs (sub-blocks past the last are zero-filled).
-        const uint32_t tx = kSub * (kABytes * (w * 2 * kBM + kBM < p.N ? 2 : 1) + n * (kBK * 2));
+        // Bytes a stage brings into both CTAs (rows and sub-blocks past the last
+        // are zero-filled).  A half tile without weight rows is copied as well: a
+        // CTA that brought nothing could be lapped by the MMAs, and a barrier two
+        // phases on looks like one not yet completed.
+        const uint32_t tx = 2 * kWSlot + kSub * n * (kBK * 2);
         for (int k = 0; k < ks; ++k) {
           // The slot is free in both CTAs once the MMAs that read it are done;
           // the leader arms its barrier with the bytes of both CTAs.
           if (!(ok = mbar_wait_hot(eb, par, &abort_flag))) break;
           if (wts && rank == 0) mbar_expect_tx(fb, tx);
-          if (live && !(wts && issued < early)) tma_load_k64_pair(dst, map, row, k * kSub, fb);
+          if (!(wts && issued < early)) tma_load_k64_pair(dst, map, row, k * kSub, fb);
           ++issued;
           dst += slot_bytes;
           eb += 8;
@@ -256,8 +258,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
       }
       if (wts && rank == 0 && pair >= units) {
         // No tile for this pair: the early copies land before the CTAs exit.
-        const uint32_t tx = kWSlot * (w_first * 2 * kBM + kBM < p.N ? 2 : 1);
-        for (int k = 0; k < early; ++k) mbar_expect_tx(smem_u32(&full_bar[k]), tx);
+        for (int k = 0; k < early; ++k) mbar_expect_tx(smem_u32(&full_bar[k]), 2 * kWSlot);
         for (int k = 0; k < early && ok; ++k) ok = mbar_wait(smem_u32(&full_bar[k]), 0, &abort_flag);
       }
       if (!ok) {
@@ -323,7 +324,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
         abort_flag = 1;
       }
       // Every MMA issued so far has completed once the drain barrier fires.
-      mma_commit_pair(smem_u32(&drain_bar));
+      mma_commit_pair(smem_u32(&drain_bar), 1);
       const unsigned long long t0 = globaltimer();
       while (!mbar_try(smem_u32(&drain_bar), 0) && globaltimer() - t0 < kTcWaitNs) {
       }

@@ -157,11 +157,12 @@ __device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint32_t a_lo, ui
       ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(acc), "r"(kHi)
       : "memory");
 }
-// Arrive on the barrier at this offset in both CTAs once the pair's MMAs issued so far are done.
-__device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
+// Arrive on the barrier at this offset in the CTAs of `ranks` (a bit mask; both
+// by default) once the pair's MMAs issued so far are done.
+__device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint16_t ranks = 3) {
   asm volatile(
       "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-      "h"(static_cast<uint16_t>(3))
+      "h"(ranks)
       : "memory");
 }
 // TMEM load of 32 columns without the wait; tmem_wait32 makes its registers usable.

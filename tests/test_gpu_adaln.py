@@ -121,6 +121,20 @@ def test_wide_block(M):
     st.close()
 
 
+@pytest.mark.parametrize("D,H,S,T", [(512, 8, 32, 32), (768, 6, 8, 264), (832, 13, 40, 40), (1280, 10, 72, 72),
+                                     (1344, 21, 24, 48), (1856, 29, 16, 16)])
+def test_row_widths_and_token_edges(M, D, H, S, T):
+    """The row kernel's builds at their widest rows and one step past them
+    (512, 768, 1280 channels; 832, 1344, 1856), which also give the projection
+    GEMMs ragged weight tiles and token tiles of 16 to 264 rows."""
+    st, cfg, ws = make_adaln_stack(M, T, D, H, 4, 2, 128, S=S, seed=13, tau0=0.72, wscale=0.03, ada_scale=0.03)
+    rng = np.random.default_rng(130)
+    xs = drift(rng.standard_normal((T, D)).astype(np.float32), rng, 3, 0.08)
+    rep, _ = run_trajectory(st, cfg, ws, xs, conds=W.conditioning(13, T // S, D, 3))
+    assert rep.layers_checked == 3
+    st.close()
+
+
 def test_full_size_d768_block(M):
     """The 12-head D 768 block of the 256px workloads: 8 samples of 256
     tokens, E 16, top-2, F 3072; one full step and two cache steps."""

@@ -413,3 +413,37 @@ def test_separate_path_step_replays_from_a_graph(M):
         torch.cuda.synchronize()
         assert torch.equal(out, want[t]), t
     st.close()
+
+
+@pytest.mark.parametrize("T", [1, 31, 32, 33, 255, 256, 257, 520])
+@pytest.mark.parametrize("D,F,S,cfg_kw", [
+    (64, 64, 0, {}),                                  # one K sub-block, a quarter of a weight tile
+    (192, 320, 1, dict(gelu_tanh=0)),                 # odd counts of K sub-blocks, ragged weight tiles
+    (256, 512, 0, dict(ffn_tile_n=64)),               # whole weight tiles, narrow token tiles
+    (320, 192, 0, dict(ffn_tile_n=192, ffn_split_k=2)),
+])
+def test_ffn_pair_kernel_edges(M, T, D, F, S, cfg_kw):
+    """Token tiles at their edges (one expert takes all T rows) and weight
+    tiles with ragged rows and K, against the SIMT path.  Both round the
+    hidden rows and the branch rows to bf16 after fp32 sums: two roundings of
+    at most 2^-9 a side, so a token's rows differ by at most 4 * 2^-9, and
+    the output's own rounding adds 2 * 2^-9."""
+    res = []
+    for impl in (M.MOECA_FFN_AUTO, M.MOECA_FFN_SIMT):
+        st, cfg, _ = make_stack(M, T, D, 1, 1, F, S=S, seed=41, bias=True, tau0=-math.inf, ffn_impl=impl, **cfg_kw)
+        x = W.round_to_bf16(np.random.default_rng(41).standard_normal((T, D)).astype(np.float32))
+        res.append(st.step(torch.from_numpy(x).cuda().to(torch.bfloat16), 0).double())
+        st.close()
+    err = (res[0] - res[1]).norm(dim=1) / res[1].norm(dim=1)
+    assert float(err.max()) < 6 * 2.0 ** -9
+
+
+def test_fp32_ffn_more_tiles_than_blocks(M):
+    """2500 rows per expert: the fp32 FFN's blocks each take several tiles."""
+    T, D, E, k, F = 5000, 64, 4, 2, 1024
+    st, cfg, ws = make_stack(M, T, D, E, k, F, seed=43, bf16=False, tau0=0.75, wscale=0.2)
+    rng = np.random.default_rng(430)
+    xs = drift(rng.standard_normal((T, D)).astype(np.float32), rng, 2, 0.05, False)
+    rep, _ = run_trajectory(st, cfg, ws, xs, bf16=False)
+    assert rep.reused > 0 and rep.recomputed > 0
+    st.close()
