@@ -109,7 +109,8 @@ struct DecideArgs {
   unsigned* epoch;            // tag of the last launch over these words, 0 before the first
 };
 // Blocks of a launch over max_tokens tokens when they are all resident at
-// once, which the exchange needs; 0 when they are not (the three kernels).
+// once, which the exchange needs, with room for a second such launch (another
+// stream's); 0 when they are not (the three kernels).
 int decide_blocks(int max_tokens, int k, int n_sms);
 cudaError_t launch_decide(const DecideArgs& a, cudaStream_t s);
 

@@ -466,7 +466,10 @@ int decide_blocks(int max_tokens, int k, int n_sms) {
     cudaGetLastError();
     return 0;
   }
-  return static_cast<long long>(occ) * n_sms >= nb ? nb : 0;
+  // Two such launches fit at once: the blocks wait for each other, so launches
+  // of two streams must not keep each other's blocks off the GPU.  (Room for
+  // four, by 64 registers a thread, spilled: top-8 / E 64 650 -> 900 us a pass.)
+  return static_cast<long long>(occ) * n_sms >= 2ll * nb ? nb : 0;
 }
 
 cudaError_t launch_decide(const DecideArgs& a, cudaStream_t s) {
