@@ -4,10 +4,11 @@
 // Phase 2: dst[list[r], :] = hmid[r, :] W2_g^T     (second half; rows land in
 //          the branch cache slot token*k+slot, or the shared-expert row)
 // Rows of group g are [offsets[g], offsets[g] + counts[g]).  The counts live
-// on the device, so the grid covers the worst case and each block finds its
-// (group, m-tile) from them; blocks past the last tile exit.  fp32 FFMA with
-// fp32 accumulation: the fp32 debug-precision path, and a cross-check of the
-// tensor-core kernel on bf16.
+// on the device: each block finds its (group, m-tile) from them.  The plain
+// kernel's grid covers the worst case, blocks past the last tile exit; the
+// pipelined fp32 kernel runs the blocks resident at once, each taking tiles in
+// turn.  fp32 FFMA with fp32 accumulation: the fp32 debug-precision path, and a
+// cross-check of the tensor-core kernel on bf16.
 #include <algorithm>
 #include <type_traits>
 
