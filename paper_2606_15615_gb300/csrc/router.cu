@@ -73,9 +73,13 @@ __global__ void __launch_bounds__(NT) router_kernel(RouterArgs a, int stage_x, i
   const int i = blockIdx.x * TB + tok;
   const bool valid = i < a.T;
   const int ntok = min(TB, a.T - static_cast<int>(blockIdx.x) * TB);
-  // Loaded before the dependency wait: the gate bias (a weight) and this
-  // token's EMA values (this layer's state, last written one step earlier by
-  // this kernel, which completed before the previous kernel could start).
+  // In a step, loaded before the dependency wait: the gate bias (a weight) and
+  // this token's EMA values (this layer's state, last written one step earlier
+  // by this kernel; the decision, FFN and combine kernels lie between, so that
+  // launch has completed).  In the allocation-free call the previous kernel can
+  // be this one on the same statistic, or a caller's that wrote it: after the
+  // wait, in flight beside the row copies.
+  if (!a.early) pdl_entry();
   float bias_pre[EPL], ema_pre[EPL];
 #pragma unroll
   for (int j = 0; j < EPL; ++j) {
@@ -83,7 +87,7 @@ __global__ void __launch_bounds__(NT) router_kernel(RouterArgs a, int stage_x, i
     bias_pre[j] = (e < E && a.b_gate) ? a.b_gate[e] : 0.f;
     ema_pre[j] = (valid && e < E) ? a.ema[static_cast<size_t>(i) * E + e] : 0.f;
   }
-  pdl_entry();
+  if (a.early) pdl_entry();
   const uint4* wsrc = static_cast<const uint4*>(a.w_gate);
   int wstride = rowv;
   const uint4* xsrc = static_cast<const uint4*>(a.x) + static_cast<size_t>(i) * rowv;

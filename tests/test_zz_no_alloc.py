@@ -128,6 +128,82 @@ def _noalloc_against_oracle(M, D, E, k, bf16):
     assert_margins(rep)
 
 
+# One shape per form of the router: groups of 1, 2, 4 and 8 lanes, 1 to 8
+# experts a lane, with the tensor cores (bf16), plain lanes (fp32), the wide
+# gate's 32-token blocks (D 1152) and rows read through L1 (D 1536).
+_FORMS = [(512, 384, 8, 2, False), (300, 64, 1, 1, True), (300, 64, 3, 2, False), (300, 128, 6, 2, True),
+          (512, 768, 16, 2, True), (300, 256, 16, 4, False), (512, 1024, 32, 4, True), (300, 1152, 64, 8, True),
+          (300, 1536, 64, 8, True), (300, 1152, 64, 8, False)]
+
+
+def _route_case(M, T, D, E, k, bf16):
+    w, x0, _ = W.tiny_layer(47, T, D, E, k, 64, dtype="bf16" if bf16 else "f32", bias=True, wscale=0.05)
+    cfg = M.moeca_config_default(n_layers=1, hidden=D, ffn=64, n_experts=E, top_k=k, max_tokens=T,
+                                 dtype=M.MOECA_BF16 if bf16 else M.MOECA_F32, tau0=0.75)
+    dt = torch.bfloat16 if bf16 else torch.float32
+    x = torch.from_numpy(np.ascontiguousarray(x0, np.float32)).cuda().to(dt)
+    return cfg, x, torch.from_numpy(w["w_gate"]).cuda().to(dt), torch.from_numpy(w["b_gate"]).cuda()
+
+
+@pytest.mark.parametrize("T,D,E,k,bf16", _FORMS)
+def test_noalloc_calls_in_a_row_are_ordered(M, T, D, E, k, bf16):
+    """Calls enqueued one right after the other on one statistic, launched and
+    replayed from a graph, give the bits of calls with a synchronisation
+    between them: each reads what the one before it wrote."""
+    cfg, x, wg, bg = _route_case(M, T, D, E, k, bf16)
+    n = 8
+    res = []
+    for wait in (True, False, False, False):
+        ema = torch.zeros((T, E), dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        outs = []
+        for _ in range(n):
+            outs.append(_noalloc(M, cfg, x, wg, bg, ema, T))
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        res.append([ema] + [o for out in outs for o in out])
+    for other in res[1:]:
+        for a, b in zip(res[0], other):
+            assert torch.equal(a, b)
+    ema = torch.zeros((T, E), dtype=torch.float32, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        for _ in range(2):
+            last = _noalloc(M, cfg, x, wg, bg, ema, T)
+    for _ in range(n // 2):
+        graph.replay()
+    torch.cuda.synchronize()
+    for a, b in zip([res[0][0]] + res[0][-3:], [ema, *last]):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("T,D,E,k,bf16", [_FORMS[0], _FORMS[4], _FORMS[7]])
+def test_noalloc_sees_what_a_kernel_just_before_it_wrote(M, T, D, E, k, bf16):
+    """The statistic, the gate matrix and its bias changed by a kernel of the
+    caller's right before the call, without a synchronisation."""
+    cfg, x, wg0, bg0 = _route_case(M, T, D, E, k, bf16)
+    res = []
+    for wait in (True, False):
+        wg, bg = wg0.clone(), bg0.clone()
+        ema = torch.zeros((T, E), dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        outs = []
+        for _ in range(4):
+            for change in (lambda: ema.mul_(0.5), lambda: wg.neg_(), lambda: bg.neg_()):
+                change()
+                if wait:
+                    torch.cuda.synchronize()
+                outs.append(_noalloc(M, cfg, x, wg, bg, ema, T))
+                if wait:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        res.append([ema] + [o for out in outs for o in out])
+    for a, b in zip(*res):
+        assert torch.equal(a, b)
+
+
 def test_noalloc_rejects_sizes_beyond_its_scratch(M):
     E = 64
     T = 16 * (32768 // E) + 1  # one 16-token block more than the scratch holds
