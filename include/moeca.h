@@ -464,9 +464,13 @@ moeca_status moeca_destroy(moeca_handle* h);
  * The first call on each device looks up that device's address of the scratch
  * array (cudaGetSymbolAddress, with that device current), so make the first
  * call on a device before any stream capture.  Every call shares the one
- * array, which keeps the last call's contents; what must start at zero is left
- * at zero by the call before.  Calls that overlap on the GPU (on different streams
- * or from different host threads) race on the scratch: serialise them.
+ * array, which keeps the last call's contents; the completion counter is left
+ * at zero by the call before and set there anew by each call.  Calls that overlap
+ * on the GPU (on different streams or from different host threads) race on the
+ * scratch: serialise them.  Overlapping calls spoil their own outputs; the next
+ * call after them is right again (a replayed capture, whose counter is only the
+ * one left to it, after one such call).  Calls on one stream are ordered: each
+ * sees what the one before, and any other work before it, wrote to its inputs.
  * Runs on the current device, asynchronously on `stream`. */
 typedef struct {
   int32_t dtype;         /* moeca_dtype of x and w_gate                       */

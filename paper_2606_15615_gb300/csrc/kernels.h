@@ -41,7 +41,8 @@ struct RouterArgs {
   float* route_w;       // [T, k]
   float* ema;           // [T, E]
   float* partials;      // [gridDim.x, E, 2]   (sum C, sum C ln C) per block
-  unsigned* done;       // last-block ticket, left at 0
+  unsigned long long* done;  // last-block ticket: blocks arrived (left at 0) below the newest tag
+  unsigned long long tag;    // 0, or above the tag of every earlier launch over this ticket
   float* tau;           // [E]
   unsigned long long* stats;
   int* status;          // device status word (or null)

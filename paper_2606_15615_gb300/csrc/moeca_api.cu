@@ -111,7 +111,8 @@ struct moeca_handle {
   int max_rows = 0;
   std::vector<LayerBuf> layers;
   float* partials = nullptr;
-  unsigned* done = nullptr;  // [0] router ticket, [1] select ticket
+  unsigned long long* router_done = nullptr;  // router ticket
+  unsigned* select_done = nullptr;            // select ticket
   int32_t* block_counts = nullptr;
   int32_t* block_offsets = nullptr;
   void* xg = nullptr;
@@ -292,7 +293,7 @@ SelectArgs select_args(const moeca_handle* h, const LayerBuf& L, int T, bool ref
   sa.cache_e = L.cache_e; sa.cache_w = L.cache_w; sa.cache_norm = L.cache_norm;
   sa.recompute = L.recompute; sa.slot = L.slot; sa.matched = L.matched; sa.token_any = L.token_any;
   sa.block_counts = h->block_counts; sa.block_offsets = h->block_offsets;
-  sa.counts = L.counts; sa.offsets = L.offsets; sa.done = h->done + 1;
+  sa.counts = L.counts; sa.offsets = L.offsets; sa.done = h->select_done;
   sa.stats = L.stats; sa.status = h->status_dev;
   return sa;
 }
@@ -558,7 +559,8 @@ moeca_status moeca_create(const moeca_config* cfg, const moeca_layer_weights* la
   const size_t nblk_router = (T + kRouterTokensPerBlock - 1) / kRouterTokensPerBlock;
   const size_t nblk_sel = (T + kSelectTokensPerBlock - 1) / kSelectTokensPerBlock;
   A((void**)&h->partials, nblk_router * E * 2 * 4);
-  A((void**)&h->done, 2 * 4);
+  A((void**)&h->router_done, 8);
+  A((void**)&h->select_done, 4);
   A((void**)&h->block_counts, nblk_sel * G * 4);
   A((void**)&h->block_offsets, nblk_sel * G * 4);
   A(&h->xg, static_cast<size_t>(h->max_rows) * D * es);
@@ -778,7 +780,7 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
     ra.renorm = c.renorm_topk; ra.beta = c.beta; ra.tau0 = tau0; ra.alpha = c.alpha;
     ra.entropy_norm = c.entropy_norm;
     ra.route_e = L.route_e; ra.route_w = L.route_w; ra.ema = L.ema;
-    ra.partials = h->partials; ra.done = h->done; ra.tau = L.tau; ra.stats = L.stats;
+    ra.partials = h->partials; ra.done = h->router_done; ra.tau = L.tau; ra.stats = L.stats;
     ra.status = h->status_dev;
     ra.early = 1;
 

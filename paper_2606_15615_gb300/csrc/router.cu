@@ -19,6 +19,7 @@
 namespace moeca {
 namespace {
 
+constexpr int kTicketBits = 28;  // blocks arrived, below the launch's tag (at most 2^30 tokens, 16 a block)
 
 // Bit-exact group reductions over the G lanes of one token (G divides 32).
 template <int G>
@@ -88,6 +89,10 @@ __global__ void __launch_bounds__(NT) router_kernel(RouterArgs a, int stage_x, i
     ema_pre[j] = (valid && e < E) ? a.ema[static_cast<size_t>(i) * E + e] : 0.f;
   }
   if (a.early) pdl_entry();
+  // A tagged launch (the allocation-free call) starts its count itself, without
+  // waiting: whichever block comes first raises the word to this launch's tag
+  // and zero blocks, so a count that overlapping launches left is not carried on.
+  if (a.tag && t == 0) atomicMax(a.done, a.tag << kTicketBits);
   const uint4* wsrc = static_cast<const uint4*>(a.w_gate);
   int wstride = rowv;
   const uint4* xsrc = static_cast<const uint4*>(a.x) + static_cast<size_t>(i) * rowv;
@@ -355,10 +360,11 @@ __global__ void __launch_bounds__(NT) router_kernel(RouterArgs a, int stage_x, i
   // The last block to arrive reduces all partials in block order.
   __threadfence();
   __syncthreads();
-  __shared__ unsigned ticket;
-  if (t == 0) ticket = atomicAdd(a.done, 1u);
+  __shared__ unsigned long long ticket;
+  if (t == 0) ticket = atomicAdd(a.done, 1ull);
   __syncthreads();
-  if (ticket != gridDim.x - 1) return;
+  constexpr unsigned long long kCountMask = (1ull << kTicketBits) - 1;
+  if ((ticket & kCountMask) != gridDim.x - 1) return;
   __threadfence();
   // Thread t sums blocks j, j + J, j + 2J, ... of expert e = t % E (J runs per
   // expert, loads independent); the J sums are then added in j order.  fp32
@@ -419,7 +425,7 @@ __global__ void __launch_bounds__(NT) router_kernel(RouterArgs a, int stage_x, i
       const bool any = lo <= hi;
       sm_lo = any ? lo : 0.f;
       sm_hi = any ? hi : 0.f;
-      *a.done = 0u;
+      *a.done = ticket & ~kCountMask;
     }
   }
   __syncthreads();
@@ -513,7 +519,7 @@ cudaError_t launch_router(const RouterArgs& a, bool bf16, cudaStream_t s) {
 namespace moeca {
 namespace {
 
-constexpr size_t kScratchHeader = 256;      // ticket at 0, counters at 64
+constexpr size_t kScratchHeader = 256;      // ticket word at 0, counters at 64
 constexpr size_t kScratchPartials = 32768;  // float2 (sum C, sum C ln C) per (block, expert)
 constexpr size_t kScratchBytes = kScratchHeader + kScratchPartials * sizeof(float2);
 constexpr int kScratchDevices = 64;
@@ -522,6 +528,7 @@ static __device__ __align__(256) unsigned char g_route_scratch[kScratchBytes];
 
 std::mutex g_scratch_mu;
 void* g_scratch_addr[kScratchDevices] = {};
+unsigned long long g_scratch_calls[kScratchDevices] = {};  // the last call's tag
 
 }  // namespace
 
@@ -548,6 +555,7 @@ extern "C" moeca_status moeca_route_noalloc(const moeca_route_args* r, void* str
   }
   if (dev < 0 || dev >= kScratchDevices) return MOECA_ERR_UNSUPPORTED;
   void* base = nullptr;
+  unsigned long long tag = 0;
   {
     std::lock_guard<std::mutex> lock(g_scratch_mu);
     if (!g_scratch_addr[dev]) {
@@ -559,13 +567,16 @@ extern "C" moeca_status moeca_route_noalloc(const moeca_route_args* r, void* str
       g_scratch_addr[dev] = p;
     }
     base = g_scratch_addr[dev];
+    tag = ++g_scratch_calls[dev];
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // The ticket starts at zero (the array is zero when loaded, and the last
-  // block of every launch sets it back), the near-tie counter only counts, and
-  // the partials are written by every block before the last block reads them.
-  // Clearing the header with a memset before each launch cost 3.5 of 14.3 us a
-  // call (512 tokens, D 384, 8 experts, fp32).
+  // The ticket's count starts at zero: the last block of every launch sets it
+  // back, and the call's tag, above every earlier call's, does so after calls
+  // that overlapped.  A replayed launch has the tag of its capture, which raises
+  // nothing past a later call's, and finds the count its predecessor set back.
+  // The near-tie counter only counts, and the partials are written by every
+  // block before the last block reads them.  A memset of the header before each
+  // launch cost 3.5 of 14.3 us a call (512 tokens, D 384, 8 experts, fp32).
   RouterArgs a{};
   a.x = r->x;
   a.w_gate = r->w_gate;
@@ -583,7 +594,8 @@ extern "C" moeca_status moeca_route_noalloc(const moeca_route_args* r, void* str
   a.route_w = r->route_w;
   a.ema = r->ema;
   a.partials = reinterpret_cast<float*>(static_cast<unsigned char*>(base) + kScratchHeader);
-  a.done = static_cast<unsigned*>(base);
+  a.done = static_cast<unsigned long long*>(base);
+  a.tag = tag;
   a.tau = r->tau;
   a.stats = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(base) + 64);
   if (launch_router(a, bf16, s) != cudaSuccess) {

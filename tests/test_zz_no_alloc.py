@@ -204,6 +204,34 @@ def test_noalloc_sees_what_a_kernel_just_before_it_wrote(M, T, D, E, k, bf16):
         assert torch.equal(a, b)
 
 
+def test_noalloc_right_again_after_calls_that_overlapped(M):
+    """Calls of different sizes on two streams at once share the scratch and
+    spoil each other's outputs (not looked at); the call after them is right."""
+    cfg, x, wg, bg = _route_case(M, *_FORMS[0])
+    T, E = cfg.max_tokens, cfg.n_experts
+    big_cfg, big_x, big_wg, big_bg = _route_case(M, 2000, 768, 16, 2, True)
+    big_ema = torch.zeros((2000, 16), dtype=torch.float32, device="cuda")
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    want = None
+    for rep in range(30):
+        if rep:
+            for s in streams:
+                s.wait_stream(torch.cuda.current_stream())
+            for _ in range(8):
+                with torch.cuda.stream(streams[0]):
+                    _noalloc(M, big_cfg, big_x, big_wg, big_bg, big_ema, 2000)
+                with torch.cuda.stream(streams[1]):
+                    _noalloc(M, cfg, x, wg, bg, torch.zeros((T, E), dtype=torch.float32, device="cuda"), T)
+            torch.cuda.synchronize()
+        ema = torch.zeros((T, E), dtype=torch.float32, device="cuda")
+        got = [ema, *_noalloc(M, cfg, x, wg, bg, ema, T)]
+        torch.cuda.synchronize()
+        if want is None:
+            want = got
+        for a, b in zip(want, got):
+            assert torch.equal(a, b), rep
+
+
 def test_noalloc_rejects_sizes_beyond_its_scratch(M):
     E = 64
     T = 16 * (32768 // E) + 1  # one 16-token block more than the scratch holds
