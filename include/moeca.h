@@ -419,14 +419,17 @@ moeca_status moeca_reset(moeca_handle* h);
 
 /* Host-side fault injection for tests of failure detection (no counterpart
  * in the paper).  MOECA_FAULT_BARRIER_STALL: the next step's fused
- * preparation kernels wait at their grid-wide exchanges for values tagged
- * with a launch number that no launch writes, as if a block never arrived;
+ * preparation kernels (or decision kernels, on a handle whose router runs by
+ * itself) wait at their grid-wide exchanges for values tagged with a launch
+ * number that no launch writes, as if a block never arrived;
  * every block gives up after about one second of %globaltimer,
  * records MOECA_ERR_TIMEOUT in the device status and skips its later phases,
  * so the step's outputs are garbage and the next call that checks the device
- * status returns MOECA_ERR_TIMEOUT until moeca_reset.  Nothing faults or
- * hangs.  Returns MOECA_ERR_UNSUPPORTED when the handle does not run the
- * fused preparation kernel (fp32, or shapes it does not fit). */
+ * status returns MOECA_ERR_TIMEOUT until moeca_reset.  After a decision kernel
+ * that gave up, the later layers' leave at once: their row lists stay what they
+ * were.  Nothing faults or hangs.  Returns MOECA_ERR_UNSUPPORTED when the
+ * handle runs neither kernel (a router by itself, with more tokens than the
+ * decision kernel's grid takes). */
 typedef enum { MOECA_FAULT_BARRIER_STALL = 1 } moeca_fault;
 moeca_status moeca_inject_fault(moeca_handle* h, int32_t kind);
 

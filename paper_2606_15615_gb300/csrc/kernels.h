@@ -102,14 +102,20 @@ cudaError_t launch_gather(const CompactArgs& a, bool bf16, cudaStream_t s);
 
 // select, compact and gather in one launch, with an exchange of the blocks' row
 // counts between them.
+struct alignas(8) DecideState {
+  unsigned epoch;             // tag of the last launch over the words, 0 before the first
+  unsigned failed;            // 1 after a launch whose exchange ran out: later launches leave at once
+};
 struct DecideArgs {
   SelectArgs sel;             // block_counts, block_offsets and done are not used
+  int rows;                   // capacity of list and xg
   int32_t* list;              // [rows]
   const void* x;              // [T, D]
   void* xg;                   // [rows, D] gathered inputs, or null: gathered later (launch_gather)
   int row_vecs;               // 16-byte vectors of a row
   unsigned long long* words;  // [blocks, G] tagged row counts
-  unsigned* epoch;            // tag of the last launch over these words, 0 before the first
+  DecideState* state;         // one for all launches over these words
+  unsigned stall;             // xor of the tag waited for: 0, or (injected) 1 << 31, a tag no launch writes
 };
 // Blocks of a launch over max_tokens tokens when they are all resident at
 // once, which the exchange needs, with room for a second such launch (another

@@ -595,7 +595,8 @@ moeca_status moeca_create(const moeca_config* cfg, const moeca_layer_weights* la
   }
   if (separate) {
     h->decide_blocks = decide_blocks(c.max_tokens, c.top_k, h->n_sms);
-    // The words, then the last launch's tag.
+    // The words, then the launches' state.
+    static_assert(sizeof(DecideState) == sizeof(unsigned long long));
     h->prep_words_n = h->decide_blocks ? static_cast<size_t>(h->decide_blocks) * G + 1 : 0;
     if (h->decide_blocks) A((void**)&h->prep_words, h->prep_words_n * 8);
   }
@@ -826,10 +827,11 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
       if ((e = timed(h, MOECA_K_ROUTER, s, [&] { return launch_router(ra, h->bf16, s); })) != cudaSuccess) break;
       if (h->decide_blocks) {
         DecideArgs da{};
-        da.sel = sa; da.list = L.list; da.x = moe_in; da.xg = xg_now;
+        da.sel = sa; da.rows = h->max_rows; da.list = L.list; da.x = moe_in; da.xg = xg_now;
         da.row_vecs = static_cast<int>(c.hidden * h->es / 16);
         da.words = h->prep_words;
-        da.epoch = reinterpret_cast<unsigned*>(h->prep_words + h->prep_words_n - 1);
+        da.state = reinterpret_cast<DecideState*>(h->prep_words + h->prep_words_n - 1);
+        da.stall = h->inject_stall ? 0x80000000u : 0u;
         e = timed(h, MOECA_K_SELECT, s, [&] { return launch_decide(da, s); });
         if (e != cudaSuccess) break;
       }
@@ -1275,7 +1277,8 @@ moeca_status moeca_reset(moeca_handle* h) {
 moeca_status moeca_inject_fault(moeca_handle* h, int32_t kind) {
   if (!h) return fail(nullptr, MOECA_ERR_INVALID_ARG, "handle is NULL");
   if (kind != MOECA_FAULT_BARRIER_STALL) return fail(h, MOECA_ERR_INVALID_ARG, "unknown fault kind");
-  if (h->prep.tokens_per_block == 0) return fail(h, MOECA_ERR_UNSUPPORTED, "no fused preparation kernel on this handle");
+  if (h->prep.tokens_per_block == 0 && h->decide_blocks == 0)
+    return fail(h, MOECA_ERR_UNSUPPORTED, "no kernel with a grid-wide exchange on this handle");
   h->inject_stall = true;
   return MOECA_OK;
 }

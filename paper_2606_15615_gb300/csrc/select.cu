@@ -270,6 +270,7 @@ __global__ void __launch_bounds__(kDecThreads) decide_kernel(DecideArgs a) {
   __shared__ int s_part[kDecThreads][2];
   __shared__ int s_pre[kMaxGroups], s_tot[kMaxGroups], s_off[kMaxGroups + 1];
   __shared__ int s_pos[kDecTokens][KMAX + 1];  // list position of each of a token's rows, -1: none
+  __shared__ unsigned s_epoch;
   __shared__ int s_fail;
   const SelectArgs& sel = a.sel;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -285,19 +286,31 @@ __global__ void __launch_bounds__(kDecThreads) decide_kernel(DecideArgs a) {
       s_cw[idx] = sel.cache_w[b0 + idx];
       s_cn[idx] = sel.cache_norm[b0 + idx];
     }
-  if (t == 0) s_fail = 0;
   pdl_entry();
   // This launch's tag: one past the last launch's, kept on the device (a
   // captured launch can be replayed), and advanced by block 0 once it has read
-  // every block's words, so every block has read it.
-  unsigned epoch = *a.epoch + 1;
-  if (epoch == 0) epoch = 1;  // 0 marks words never written
+  // every block's words.  A block publishes after the barrier below, so block 0
+  // then knows that every block has read its tag.
+  // A launch whose exchange failed leaves the tag as it was or not, and blocks
+  // of it may still start: from then on no block publishes, reads words or
+  // writes lists, in this launch or a later one (any layer's), until
+  // moeca_reset clears the words.  Row counts of different launches under one
+  // tag would send list and row writes past their buffers.
+  unsigned long long state = 0;  // {epoch, failed}, in flight beside the loads below
+  if (t == 0) state = ld_word(reinterpret_cast<const unsigned long long*>(a.state));
   for (int idx = t; idx < ntok * k; idx += kDecThreads) {
     s_re[idx] = sel.route_e[b0 + idx];
     s_rw[idx] = sel.route_w[b0 + idx];
   }
   if (t < E) s_tau[t] = sel.tau[t];
+  if (t == 0) {
+    const unsigned e = static_cast<unsigned>(state) + 1;
+    s_epoch = e ? e : 1;  // 0 marks words never written
+    s_fail = static_cast<int>(state >> 32);
+  }
   __syncthreads();
+  if (s_fail) return;
+  const unsigned epoch = s_epoch;
 
   TokenDecisionT<KMAX> d;
   if (warp == 0) {
@@ -352,7 +365,7 @@ __global__ void __launch_bounds__(kDecThreads) decide_kernel(DecideArgs a) {
       const int lo = static_cast<int>(static_cast<long long>(j) * nb / R);
       const int hi = static_cast<int>(static_cast<long long>(j + 1) * nb / R);
       ok = read_tagged<16>(
-          a.words, hi - lo, [&](int q) { return static_cast<size_t>(lo + q) * G + g; }, epoch,
+          a.words, hi - lo, [&](int q) { return static_cast<size_t>(lo + q) * G + g; }, epoch ^ a.stall,
           globaltimer() + kDecWaitNs, [&](int q, uint32_t v) {
             const int c = static_cast<int>(v);
             if (lo + q < me) pre += c;
@@ -361,6 +374,7 @@ __global__ void __launch_bounds__(kDecThreads) decide_kernel(DecideArgs a) {
     }
     if (!ok) {
       report_status(sel.status, kStatusWaitTimeout, 620);
+      *static_cast<volatile unsigned*>(&a.state->failed) = 1u;
       s_fail = 1;
     }
     s_part[t][0] = pre;
@@ -396,6 +410,13 @@ __global__ void __launch_bounds__(kDecThreads) decide_kernel(DecideArgs a) {
     if (lane == 0) s_off[G] = carry;
     __syncwarp();
     // The block's row lists, ascending tokens within each group.
+    bool over = false;  // a place past the list's end (its row is left out)
+    auto in_list = [&](int pos, int row) {
+      const bool in = pos < a.rows;
+      over |= !in;
+      if (in) a.list[pos] = row;
+      return in ? pos : -1;
+    };
     const unsigned lt = (1u << lane) - 1u;
     const int i = tok0 + lane;
 #pragma unroll
@@ -403,21 +424,18 @@ __global__ void __launch_bounds__(kDecThreads) decide_kernel(DecideArgs a) {
       int pos = -1;
       if (d.rec[p]) {
         const int g = d.e[p];
-        pos = s_off[g] + s_pre[g] + __popc(s_bal[g] & lt);
-        a.list[pos] = i * k + d.sl[p];
+        pos = in_list(s_off[g] + s_pre[g] + __popc(s_bal[g] & lt), i * k + d.sl[p]);
       }
       s_pos[lane][p] = pos;
     }
     int pos = -1;
-    if (d.shared_row) {
-      pos = s_off[E] + s_pre[E] + __popc(s_bal[E] & lt);
-      a.list[pos] = i;
-    }
+    if (d.shared_row) pos = in_list(s_off[E] + s_pre[E] + __popc(s_bal[E] & lt), i);
     s_pos[lane][KMAX] = pos;
+    if (over) report_status(sel.status, kStatusBadIndex, 6200000 + i);
   }
   __syncthreads();
   if (blockIdx.x == 0) {
-    if (t == 0) *a.epoch = epoch;
+    if (t == 0) a.state->epoch = epoch;
     for (int g = t; g < G; g += kDecThreads) sel.counts[g] = s_tot[g];
     for (int g = t; g <= G; g += kDecThreads) sel.offsets[g] = s_off[g];
   }

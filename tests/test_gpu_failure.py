@@ -5,6 +5,9 @@
   after about a second, the device status records a timeout, the next call
   reports MOECA_ERR_TIMEOUT, and moeca_reset brings the handle back to
   results identical to a fresh handle's.
+* The same for the decision kernel's exchange on a handle whose router runs by
+  itself, where the later layers' launches must leave the failed one's words
+  alone.
 * A device allocation that cannot succeed is reported as MOECA_ERR_OOM and
   leaves nothing behind: a normal handle can be created right after.
 * A cached expert id out of range, written by the host, is reported as a
@@ -70,6 +73,62 @@ def test_barrier_stall_times_out_and_reset_recovers(M):
 
     M.moeca_reset(st.handle)
     st.stats()                 # the status is clear again
+    got = _run(st, xs)
+    for a, b in zip(got, expected):
+        assert torch.equal(a, b)
+    st.close()
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+def test_decision_stall_leaves_later_layers_alone_and_reset_recovers(M, bf16):
+    """The decision kernel of a handle whose router runs by itself (fp32; bf16
+    on the CUDA-core FFN), two layers: the first layer's exchange gives up,
+    the second layer's launch, which shares the exchange's words, leaves at
+    once with its lists as they were, and moeca_reset recovers."""
+    import time
+    import torch
+    from paper_2606_15615_gb300.workloads import tiny_layer
+    T, D, E, k, F = 300, 128, 8, 2, 192
+    ws, dt = [], torch.bfloat16 if bf16 else torch.float32
+    for l in range(2):
+        w, x0, rng = tiny_layer(8 + l, T, D, E, k, F, dtype="bf16" if bf16 else "f32", wscale=0.05)
+        ws.append(w)
+    cfg = M.moeca_config_default(n_layers=2, hidden=D, ffn=F, n_experts=E, top_k=k, max_tokens=T, tau0=0.75,
+                                 dtype=M.MOECA_BF16 if bf16 else M.MOECA_F32, ffn_impl=M.MOECA_FFN_SIMT)
+    xs = [x0]
+    for _ in range(2):
+        xs.append((xs[-1] + 0.05 * rng.standard_normal(x0.shape)).astype(np.float32))
+    xs = [torch.from_numpy(x).cuda().to(dt) for x in xs]
+    ref = M.Stack(cfg, ws)
+    expected = _run(ref, xs)
+    assert 0 < ref.stats()["reused"] < ref.stats()["cache_step_branches"]
+    ref.close()
+
+    st = M.Stack(cfg, ws)
+    st.step(xs[0], 0)
+    keys = ("recompute", "slot", "counts", "offsets", "list")
+    before = [{q: st.get_trace(l, T)[q].clone() for q in keys} for l in range(2)]
+    torch.cuda.synchronize()
+    M.moeca_inject_fault(st.handle, M.MOECA_FAULT_BARRIER_STALL)
+    t0 = time.monotonic()
+    st.step(xs[1], 1)
+    torch.cuda.synchronize()
+    assert 0.9 < time.monotonic() - t0 < 1.7   # one wait, not one a layer
+    after = [st.get_trace(l, T) for l in range(2)]
+    torch.cuda.synchronize()
+    for q in ("counts", "offsets", "list"):    # layer 0 decided, but placed no row
+        assert torch.equal(before[0][q], after[0][q]), q
+    for q in keys:
+        assert torch.equal(before[1][q], after[1][q]), q
+    with pytest.raises(M.MoecaError) as err:
+        st.stats()
+    assert err.value.status == M.MOECA_ERR_TIMEOUT
+    with pytest.raises(M.MoecaError) as err:
+        st.step(xs[2], 2)
+    assert err.value.status == M.MOECA_ERR_TIMEOUT
+
+    M.moeca_reset(st.handle)
+    st.stats()
     got = _run(st, xs)
     for a, b in zip(got, expected):
         assert torch.equal(a, b)
