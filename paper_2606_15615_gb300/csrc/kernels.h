@@ -46,8 +46,6 @@ struct RouterArgs {
   float* tau;           // [E]
   unsigned long long* stats;
   int* status;          // device status word (or null)
-  int early;            // 1: b_gate and ema may be read before the previous kernel on the stream has
-                        // ended (neither it nor the caller just wrote them)
 };
 cudaError_t launch_router(const RouterArgs& a, bool bf16, cudaStream_t s);
 

@@ -783,7 +783,6 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
     ra.route_e = L.route_e; ra.route_w = L.route_w; ra.ema = L.ema;
     ra.partials = h->partials; ra.done = h->router_done; ra.tau = L.tau; ra.stats = L.stats;
     ra.status = h->status_dev;
-    ra.early = 1;
 
     SelectArgs sa = select_args(h, L, T, refresh);
 
