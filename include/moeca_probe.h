@@ -11,6 +11,9 @@
  * row written): at tens of MB a launch's ramp and drain are a sizeable part
  * of its time, so the large-copy HBM peak is out of reach for any kernel of
  * that size, and this figure says how far.
+ *
+ * moeca_probe_hold occupies SMs for a stated time, so that tests can run the
+ * library's kernels on a GPU they do not have to themselves.
  */
 #ifndef MOECA_PROBE_H_
 #define MOECA_PROBE_H_
@@ -48,6 +51,15 @@ int32_t moeca_probe_ffma(int32_t device, int32_t iterations, double* tflops, dou
  * included). */
 int32_t moeca_probe_stream(int32_t device, int64_t n_tokens, int32_t rows, int32_t row_bytes, int32_t reps,
                            double* gbs, double* us);
+
+/* Keep part of CUDA device `device` busy for a while, as another program's
+ * kernels would: `blocks` one-warp blocks in clusters of two (so that they take
+ * pairs of SMs), each holding `smem_bytes` of shared memory (above half an SM's:
+ * one block per SM) and sleeping until `us` microseconds have passed.  They wait
+ * for nothing else.  Enqueued on `stream` (a cudaStream_t), asynchronous.
+ * Constraints: blocks even, 2 <= blocks <= the SM count, 0 <= smem_bytes <= 200 KB, 1 <= us <= 2000000.  Returns 0, or -1 (bad
+ * device, a constraint broken) / -3 (a CUDA call failed). */
+int32_t moeca_probe_hold(int32_t device, int32_t blocks, int32_t smem_bytes, int32_t us, void* stream);
 
 #ifdef __cplusplus
 }

@@ -108,8 +108,7 @@ struct TcArgs {
   int* tile_sem;   // split-K arrival counters, one per epilogue warp of a half tile, left at 0
   int* dep;        // per token tile {phase-1 half tiles stored, phase-2 CTAs started}, left at 0
   int dep_pairs;   // capacity of dep (pairs)
-  int* work;       // next unit ticket (units past each pair's first go to whoever asks); the kernel
-                   // after this one re-arms it to 0 (launch_ffn_tc's contract)
+  int* work;       // next unit ticket; the kernel after this one re-arms it to 0 (launch_ffn_tc's contract)
   int* status;
 };
 
@@ -311,12 +310,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ uint32_t tmem_base_sh;
   __shared__ Groups gr;
   __shared__ int nmax_sh;
+  __shared__ __align__(8) uint64_t ticket_bar;  // the peer's: the pair's first ticket is there
+  __shared__ int ticket_sh;
   __shared__ volatile int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = a.G;
   const uint32_t rank = cluster_rank();
-  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
   // Everything that does not read the previous kernel's output happens
   // before the programmatic-dependency wait: barriers, TMEM, map prefetch.
@@ -331,6 +331,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(smem_u32(&tempty_bar[s]), 2 * kEpiWarps);
     }
     mbar_init(smem_u32(&drain_bar), 1);
+    mbar_init(smem_u32(&ticket_bar), 1);
+    mbar_expect_tx(smem_u32(&ticket_bar), 4);
     for (int q = 0; q < kUQ; ++q) {
       mbar_init(smem_u32(&uq_full[q]), 1);
       mbar_init(smem_u32(&pub_bar[q]), kEpiWarps);
@@ -360,8 +362,26 @@ __global__ void __launch_bounds__(kThreads, 1)
                  "l"(a.counts), "l"(a.offsets), "l"(a.list), "l"(a.hmid), "l"(a.dep), "l"(a.cache_h), "l"(a.work),
                  "r"(a.E), "r"(a.dep_pairs));
   }
-  cluster_arrive();
+  // The pair's first ticket.  The counter was re-armed by a combine that lies
+  // before the previous kernel, which has passed its own wait.  Drawn this
+  // early by a warp that has nothing to release, the ticket costs at most 0.5 us
+  // a launch against first units fixed to the pair's index (D 768, 2048 tokens,
+  // 4 layer steps 278.7 -> 280.7 us; 0.9 us with the draw in warp 0, and as much
+  // with fixed first units that other pairs can take: code that runs first
+  // after the wait is fetched while the weights stream in).
+  int drawn = 0;
+  if (warp == 3) {
+    if (lane == 0 && rank == 0) drawn = atomicAdd(a.work, 1);
+    cluster_arrive_relaxed();
+  } else {
+    cluster_arrive();
+  }
   cluster_wait();  // both CTAs' barriers are initialised
+  if (warp == 3 && lane == 0 && rank == 0) {
+    // To both CTAs' weight producers.
+    st_async_cluster(cluster_addr(smem_u32(&ticket_sh), 1), drawn, cluster_addr(smem_u32(&ticket_bar), 1));
+    ticket_sh = drawn;
+  }
   Phase p0, p1;
   p0.nw = (a.N[0] + 255) >> 8;
   p1.nw = (a.N[1] + 255) >> 8;
@@ -438,12 +458,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t uqe0 = cluster_addr(smem_u32(&uq_empty[0]), 0);
       const uint32_t uqf1 = cluster_addr(smem_u32(&uq_full[0]), 1);
       const uint32_t uq1 = cluster_addr(smem_u32(&uq[0]), 1);
-      // Units: the pair's index first, then tickets from the shared counter,
-      // in increasing order (so phase 1 before phase 2 here too).  The leader
-      // decodes each and passes it to the other roles of both CTAs through the
-      // unit queue; a negative word ends it.  The ticket is drawn four stages
-      // before the end of a unit and passed on one stage before it, so that
-      // neither round trip leaves the ring idle.
+      // Units: tickets from the shared counter, in increasing order (so phase 1
+      // before phase 2 here too).  A pair owns a unit only by drawing it, the
+      // first one included: a pair that another stream's kernels keep off the
+      // GPU holds up nobody's phase 2.  The leader decodes each unit and passes
+      // it to the other roles of both CTAs through the unit queue; a negative
+      // word ends it.  The next ticket is drawn four stages before the end of a
+      // unit and passed on one stage before it, so that neither round trip
+      // leaves the ring idle.
       auto push = [&](const int4& v) -> bool {
         if (!mbar_wait(smem_u32(&uq_empty[qs]), qpar ^ 1u, &abort_flag)) return false;
         uq[qs] = v;
@@ -456,8 +478,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         return true;
       };
-      // The first unit is known without the queue.
-      int4 cur = unit_word(pair, total, p0, p1, gr, G);
+      // The first unit does without the queue: the peer decodes its ticket too.
+      if (!leader)
+        ok = mbar_try_cluster(smem_u32(&ticket_bar), 0) || mbar_wait_cluster(smem_u32(&ticket_bar), 0, &abort_flag);
+      int ticket = *static_cast<volatile int*>(&ticket_sh);
+      int4 cur = unit_word(ticket, total, p0, p1, gr, G);
       if (leader) ok = push(cur);
       for (bool first = true; ok; first = false) {
         if (!leader) {
@@ -484,7 +509,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int k0 = t.sp * ks / S, k1 = (t.sp + 1) * ks / S;  // stages of this unit
         // Bytes a stage brings into both CTAs (sub-blocks past the last are zero-filled).
         const uint32_t stage_tx = kSub * (2 * kABytes + t.n * (kBK * 2));
-        int ticket = 0;
         int k = k0;
         for (int part = 0; part < 3 && ok; ++part) {
           // Up to four stages before the end, up to one, to the end.
@@ -507,7 +531,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
           }
           if (leader && ok) {
-            if (part == 0) ticket = n_pairs + atomicAdd(a.work, 1);
+            if (part == 0) ticket = atomicAdd(a.work, 1);
             if (part == 1) {
               cur = unit_word(ticket, total, p0, p1, gr, G);
               ok = push(cur);

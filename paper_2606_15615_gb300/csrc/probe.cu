@@ -1,6 +1,7 @@
 // Measurement probes (include/moeca_probe.h): the fp32 FMA throughput (the
 // roofline of the fp32 debug path's SIMT expert FFN) and the rate a plain
-// streaming kernel reaches at the combine's size and shape.
+// streaming kernel reaches at the combine's size and shape; and a kernel that
+// only occupies SMs.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -63,6 +64,17 @@ __global__ void l2_read_kernel(const uint4* __restrict__ p, size_t n, uint4* sin
     a ^= v.x ^ v.y ^ v.z ^ v.w;
   }
   if (a == 0x9e3779b9u) sink->x = a;  // never true for the zeroed buffer; keeps the loads
+}
+
+// Sleeps until `us` microseconds have passed; the turns of the loop are bounded too.
+__global__ void hold_kernel(int us) {
+  unsigned long long t0, t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+  for (int it = 0; it < 8 * us; ++it) {
+    __nanosleep(1000);  // up to twice that, or less
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    if (t - t0 >= 1000ull * us) break;
+  }
 }
 
 template <int ROWS>
@@ -177,4 +189,33 @@ extern "C" int32_t moeca_probe_ffma(int32_t device, int32_t iterations, double* 
   *ms = t;
   *tflops = 2.0 * fmas / (t * 1e-3) / 1e12;
   return 0;
+}
+
+extern "C" int32_t moeca_probe_hold(int32_t device, int32_t blocks, int32_t smem_bytes, int32_t us, void* stream) {
+  int ndev = 0, n_sms = 0;
+  if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev) {
+    cudaGetLastError();
+    return -1;
+  }
+  if (blocks < 2 || blocks % 2 || smem_bytes < 0 || smem_bytes > 200 * 1024 || us < 1 || us > 2000000) return -1;
+  bool ok = cudaSetDevice(device) == cudaSuccess &&
+            cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, device) == cudaSuccess;
+  if (ok && blocks > n_sms) return -1;
+  ok = ok && cudaFuncSetAttribute(hold_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) == cudaSuccess;
+  if (ok) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(32);
+    cfg.dynamicSmemBytes = smem_bytes;
+    cfg.stream = static_cast<cudaStream_t>(stream);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    ok = cudaLaunchKernelEx(&cfg, hold_kernel, us) == cudaSuccess;
+  }
+  if (!ok) cudaGetLastError();
+  return ok ? 0 : -3;
 }

@@ -144,6 +144,7 @@ def _load():
                                           C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_double)]),
         "moeca_ddpm_step": (C.c_int, [C.POINTER(moeca_ddpm_args), C.c_void_p]),
         "moeca_probe_ffma": (C.c_int32, [C.c_int32, C.c_int32, C.POINTER(C.c_double), C.POINTER(C.c_double)]),
+        "moeca_probe_hold": (C.c_int32, [C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_void_p]),
         "moeca_probe_stream": (C.c_int32, [C.c_int32, C.c_int64, C.c_int32, C.c_int32, C.c_int32,
                                            C.POINTER(C.c_double), C.POINTER(C.c_double)]),
     }
@@ -328,6 +329,13 @@ def moeca_probe_ffma(device: int = 0, iterations: int = 1 << 16) -> tuple:
     if st != 0:
         raise MoecaError(st, "moeca_probe_ffma")
     return tf.value, ms.value
+
+
+def moeca_probe_hold(device: int, blocks: int, smem_bytes: int, us: int, stream: int) -> None:
+    """Keep ``blocks`` SMs' shared memory busy for ``us`` microseconds (include/moeca_probe.h)."""
+    st = LIB.moeca_probe_hold(device, blocks, smem_bytes, us, stream)
+    if st != MOECA_OK:
+        raise MoecaError(st, "moeca_probe_hold")
 
 
 def moeca_probe_stream(device: int, n_tokens: int, rows: int, row_bytes: int, reps: int = 15) -> tuple:

@@ -7,6 +7,7 @@ bf16 paths, a shared expert with skewed routing, the fine-grained 64-expert
 top-8 shape, each reading switch, and the degenerate cases.
 """
 import math
+import time
 
 import numpy as np
 import pytest
@@ -436,6 +437,33 @@ def test_ffn_pair_kernel_edges(M, T, D, F, S, cfg_kw):
         st.close()
     err = (res[0] - res[1]).norm(dim=1) / res[1].norm(dim=1)
     assert float(err.max()) < 6 * 2.0 ** -9
+
+
+@pytest.mark.parametrize("E,F", [(8, 3072), (8, 1024), (2, 256)])
+def test_ffn_pairs_kept_off_the_gpu_hold_up_nobody(M, E, F):
+    """Half of the SMs held by another stream's kernel for longer than the
+    FFN's bounded waits: the resident CTA pairs do the units of the others, so
+    no phase-2 unit waits for a pair that is not there, and the step gives its
+    usual bits.  First GEMM units (96, 32, 2) above and below the pairs' number."""
+    T, D, k = 256, 768, 2
+    x = torch.from_numpy(W.round_to_bf16(np.random.default_rng(44).standard_normal((T, D)).astype(np.float32)))
+    x = x.cuda().to(torch.bfloat16)
+    n_sms = torch.cuda.get_device_properties(0).multi_processor_count
+    outs = []
+    side = torch.cuda.Stream()
+    for hold in (False, True):
+        st, cfg, _ = make_stack(M, T, D, E, k, F, seed=44, refresh_period=1)
+        for t in range(2):
+            torch.cuda.synchronize()
+            if hold and t:
+                M.moeca_probe_hold(0, n_sms // 4 * 2, 160 * 1024, 1300000, side.cuda_stream)
+                time.sleep(0.02)
+            outs.append(st.step(x, t))
+        torch.cuda.synchronize()
+        st.stats()  # raises if a wait ran out
+        st.close()
+    for o in outs[1:]:
+        assert torch.equal(o, outs[0])
 
 
 def test_fp32_ffn_more_tiles_than_blocks(M):
