@@ -24,6 +24,11 @@
  *  - Weights and activation buffers are BORROWED: the caller owns them and
  *    keeps them alive (weights for the handle's lifetime).  The library owns
  *    every state and workspace buffer it allocates in moeca_create().
+ *  - Weights may be changed in place between steps, in stream order.  One of
+ *    them, w_gate on bf16 stacks without AdaLN, may be read while the work
+ *    enqueued right before moeca_step on its stream is ending: if that is the
+ *    kernel which changed it, synchronise the stream first (a copy or an event
+ *    wait in between orders it as well).
  *  - Every function returns a moeca_status; none throws or aborts.  Kernels
  *    never trap: a device-side problem (an index out of range, a bounded wait
  *    that ran out) is written to a status word that the next moeca_step()

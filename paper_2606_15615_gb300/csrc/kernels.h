@@ -279,6 +279,8 @@ struct ProjArgs {
   void* vt_out;           // kProjQKV: [D, n_tok] v transposed
   const float* gate;      // kProjResidualGated: u = x + gate * a, the gate row of token t at
   int gate_ld, seq;       //   gate + (t / seq) * gate_ld (AdaLN block)
+  int first;              // 1: a step's first launch; the kernel before it is the caller's and may have
+                          //   written the weights, so that none load before the dependency wait
   int* status;
 };
 cudaError_t launch_proj_tc(const ProjArgs& a, int n_sms, cudaStream_t s);

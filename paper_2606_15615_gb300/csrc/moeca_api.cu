@@ -739,6 +739,7 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
     }
     if (attn_full) {
       // Every token's attention output, before the router sees u = x + a.
+      qa.first = l == 0 && !ada;
       if (ada) {
         AdaLnArgs ha = la;
         ha.h_out = h->ada_h;

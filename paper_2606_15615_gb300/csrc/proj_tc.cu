@@ -91,6 +91,7 @@ struct ProjParams {
   __nv_bfloat16* vt_out;     // kProjQKV: [D, n_tok]
   const float* gate;         // kProjResidualGated: gate row of token t at gate + (t / seq) * gate_ld
   int gate_ld, seq;
+  int first;                 // 1: no weights before the dependency wait (see ProjArgs)
   int* status;
 };
 
@@ -200,7 +201,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
   // The weights of the first tile's first stages load before the dependency
   // wait: which they are does not depend on the row count.  Their bytes
   // complete on the stages' barriers, which the leader arms after the wait.
-  const int early = min(kEarly, ks), w_first = pair % nw;
+  // Not in a step's first launch: a caller's kernel right before it that wrote
+  // the weights has ended then, but only the wait makes its writes visible.
+  const int early = p.first ? 0 : min(kEarly, ks), w_first = pair % nw;
   if (warp == 0 && lane == 0) {
     const int feat = w_first * 2 * kBM + static_cast<int>(rank) * kBM;
     const uint32_t full0 = cluster_addr(smem_u32(&full_bar[0]), 0);
@@ -498,6 +501,7 @@ cudaError_t launch_proj_tc(const ProjArgs& a, int n_sms, cudaStream_t s) {
   p.k_out = static_cast<__nv_bfloat16*>(a.k_out);
   p.vt_out = static_cast<__nv_bfloat16*>(a.vt_out);
   p.gate = a.gate; p.gate_ld = a.gate_ld; p.seq = a.seq;
+  p.first = a.first;
   p.status = a.status;
   // At most one pair per tile of the narrowest width.
   const int nw = (a.N + 2 * kBM - 1) / (2 * kBM);

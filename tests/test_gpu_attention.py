@@ -248,3 +248,33 @@ def test_wide_block_separate_path(M):
     rep, _ = run_trajectory(st, cfg, ws, xs)
     assert rep.reused > 0 and rep.attn_rows > T
     st.close()
+
+
+def test_full_step_sees_projection_weights_a_kernel_just_before_wrote(M):
+    """w_qkv and w_o changed in place by kernels of the caller's, the last one
+    right before a full step (whose first launch reads w_qkv), with and without
+    a synchronisation in between: the same bits."""
+    T, D, H, S = 512, 768, 12, 256
+    rng = np.random.default_rng(160)
+    x = torch.from_numpy(W.round_to_bf16(rng.standard_normal((T, D)).astype(np.float32))).cuda().to(torch.bfloat16)
+    outs = []
+    for wait in (True, False):
+        w, _, _ = W.tiny_layer(16, T, D, 8, 2, 256, dtype="bf16", wscale=0.05)
+        w.update(W.tiny_attn(16, D, dtype="bf16", wscale=0.05))
+        w = {q: torch.from_numpy(v).cuda().to(torch.bfloat16) if q in ("w_qkv", "w_o") else v for q, v in w.items()}
+        cfg = M.moeca_config_default(n_layers=1, hidden=D, ffn=256, n_experts=8, top_k=2, max_tokens=T, n_heads=H,
+                                     seq_len=S, dtype=M.MOECA_BF16, tau0=0.72, refresh_period=1)
+        st = M.Stack(cfg, [w])
+        assert w["w_qkv"].data_ptr() in {k.data_ptr() for k in st._keep}  # the caller's tensor itself
+        for t in range(6):
+            w["w_o"].neg_()
+            w["w_qkv"].mul_(-0.5 if t % 2 else -2.0)
+            if wait:
+                torch.cuda.synchronize()
+            outs.append(st.step(x, t))
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        st.close()
+    for a, b in zip(outs[:6], outs[6:]):
+        assert torch.equal(a, b)
