@@ -150,8 +150,11 @@ typedef struct {
                                  routes and decides, its blocks bring up to this many MB of the
                                  layer's routed first-GEMM weights (W1, from expert 0 on, the order
                                  in which the grouped GEMM takes them) into L2, so that the GEMM's
-                                 first phase reads them from L2 instead of HBM.  A cache hint: the
-                                 results do not depend on it.  0 = none; default 16; at most 4096 */
+                                 first phase reads them from L2 instead of HBM.  The whole amount at
+                                 64 or more blocks (from 2017 tokens on, in blocks of 32); with
+                                 fewer, a 64th of it per block (2 MB of 16 at 256 tokens).  A cache
+                                 hint: the results do not depend on it.  0 = none; default 16; at
+                                 most 4096 */
 } moeca_config;
 
 /* Fill `cfg` with the defaults above and the paper's hyper-parameters

@@ -61,6 +61,11 @@ int32_t moeca_probe_stream(int32_t device, int64_t n_tokens, int32_t rows, int32
  * device, a constraint broken) / -3 (a CUDA call failed). */
 int32_t moeca_probe_hold(int32_t device, int32_t blocks, int32_t smem_bytes, int32_t us, void* stream);
 
+/* Bytes of a layer's routed first-GEMM weights (w1_bytes in all) that a launch
+ * of the fused preparation kernel with `blocks` blocks brings into L2 under
+ * moeca_config.weight_prefetch_mb = setting_mb.  Runs on the host. */
+int64_t moeca_probe_prefetch_bytes(int64_t w1_bytes, int32_t setting_mb, int32_t blocks);
+
 #ifdef __cplusplus
 }
 #endif

@@ -211,6 +211,9 @@ struct PrepShape {
   size_t smem;            // dynamic shared memory per block
   bool attn;              // the DiT-MoE block build of the kernel
 };
+// Bytes of the routed W1 that a launch of `blocks` blocks brings into L2 under
+// weight_prefetch_mb = setting_mb: a multiple of 16.
+size_t prep_prefetch_bytes(size_t w1_bytes, int setting_mb, int blocks);
 constexpr size_t kPrepSmemMax = 200 * 1024;
 // attn: the DiT-MoE block build; stage_a: its blocks also stage the cached
 // attention rows (a block without AdaLN, whose router input is x + a^{t0}).

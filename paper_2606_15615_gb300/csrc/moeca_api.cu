@@ -314,10 +314,11 @@ PrepArgs prep_args_plain(const moeca_handle* h, const LayerBuf& L, const void* m
   pa.part_words = h->prep_words; pa.count_words = h->prep_words + h->prep_count_off;
   pa.counts = L.counts; pa.offsets = L.offsets; pa.list = L.list;
   pa.xg = xg; pa.stats = L.stats; pa.status = h->status_dev;
-  // The head of the routed W1, in the GEMM's expert order (a whole number of 16-byte units).
+  // The head of the routed W1, in the GEMM's expert order.
   const size_t w1_bytes = static_cast<size_t>(c.n_experts) * c.ffn * c.hidden * h->es;
+  const int tb = h->prep.tokens_per_block;
   pa.l2_pf = L.w.w1;
-  pa.l2_pf_bytes = std::min(w1_bytes, static_cast<size_t>(c.weight_prefetch_mb) << 20) & ~size_t(15);
+  pa.l2_pf_bytes = prep_prefetch_bytes(w1_bytes, c.weight_prefetch_mb, (T + tb - 1) / tb);
   return pa;
 }
 

@@ -30,6 +30,8 @@
 // The results are those of router_kernel + select_kernel + compact_kernel,
 // which remain the path for fp32, for shapes whose staging does not fit in
 // shared memory, and for grids that cannot be co-resident.
+#include <algorithm>
+
 #include "common.cuh"
 #include "exchange.cuh"
 #include "kernels.h"
@@ -54,7 +56,6 @@ constexpr bool kAttn = MOECA_PREP_ATTN != 0;
 constexpr int kThreads = 128;
 constexpr int kMaxGroups = kMaxExperts + 1;
 constexpr unsigned long long kBarrierNs = 1000000000ull;
-constexpr size_t kPrefetchPerBlock = 256 * 1024;  // 16 MB over 64 blocks (2048 tokens)
 
 template <int G>
 __device__ __forceinline__ float grp_max(float v) {
@@ -267,12 +268,8 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(PrepArgs a) {
   // The grouped GEMM after this kernel reads the routed W1 first, expert by
   // expert.  HBM is nearly idle while the routing, the exchanges and the
   // decisions run, so the blocks bring its head into L2 now (a hint, issued
-  // once the block's own rows have landed so as not to delay them).  A block
-  // ends only when its prefetches have, so each takes at most
-  // kPrefetchPerBlock: 8 blocks with 2 MB each took 30 us instead of 23.
-  if (warp == 0 && a.l2_pf_bytes)
-    l2_prefetch_share(a.l2_pf, min(a.l2_pf_bytes, static_cast<size_t>(gridDim.x) * kPrefetchPerBlock), blockIdx.x,
-                      gridDim.x, lane);
+  // once the block's own rows have landed so as not to delay them).
+  if (warp == 0 && a.l2_pf_bytes) l2_prefetch_share(a.l2_pf, a.l2_pf_bytes, blockIdx.x, gridDim.x, lane);
   if constexpr (kAttn) {
     if (add_a) {
       // u = x + a^{t0}: the router input, the rows the FFN gathers, and the
@@ -865,6 +862,14 @@ cudaError_t launch_prep_plain(const PrepArgs& a, const PrepShape& p, cudaStream_
 }
 
 #if !MOECA_PREP_ATTN
+// A block ends only when its prefetches have, so a launch of few blocks takes
+// less: each block a 64th of the setting (256 KB at 16 MB; 8 blocks with 2 MB
+// each took 30 us instead of 23).
+size_t prep_prefetch_bytes(size_t w1_bytes, int setting_mb, int blocks) {
+  const size_t all = static_cast<size_t>(setting_mb) << 20;
+  return std::min(w1_bytes, all / 64 * std::min(blocks, 64)) & ~size_t(15);
+}
+
 PrepShape prep_plan(int D, int E, int k, int max_tokens, int n_sms, bool attn, bool stage_a) {
   return attn ? prep_plan_attn(D, E, k, max_tokens, n_sms, stage_a) : prep_plan_plain(D, E, k, max_tokens, n_sms);
 }

@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "kernels.h"
 #include "moeca_probe.h"
 
 namespace {
@@ -218,4 +219,9 @@ extern "C" int32_t moeca_probe_hold(int32_t device, int32_t blocks, int32_t smem
   }
   if (!ok) cudaGetLastError();
   return ok ? 0 : -3;
+}
+
+extern "C" int64_t moeca_probe_prefetch_bytes(int64_t w1_bytes, int32_t setting_mb, int32_t blocks) {
+  if (w1_bytes < 0 || setting_mb < 0 || blocks < 0) return -1;
+  return static_cast<int64_t>(moeca::prep_prefetch_bytes(static_cast<size_t>(w1_bytes), setting_mb, blocks));
 }

@@ -129,3 +129,15 @@ def test_ddpm_schedule_matches_the_oracle(lib):
                                x_t=4096, eps=4096, z=4096, x_prev=4096)
     with pytest.raises(lib.MoecaError):          # n not a multiple of 8: refused before any launch
         lib.moeca_ddpm_step(args)
+
+
+def test_weight_prefetch_setting_counts_at_every_launch_size(lib):
+    """weight_prefetch_mb: the whole setting from 64 blocks on, a 64th of it per
+    block below, never more than the weights; larger settings bring more."""
+    f = lib.LIB.moeca_probe_prefetch_bytes
+    MB, w1 = 1 << 20, 3000 << 20
+    assert [f(w1, 16, b) // MB for b in (8, 32, 64, 128)] == [2, 8, 16, 16]
+    for b in (1, 8, 63, 64, 200):
+        got = [f(w1, mb, b) for mb in (0, 1, 16, 17, 64, 1024, 4096)]
+        assert got[0] == 0 and got == sorted(set(got)) and all(g % 16 == 0 for g in got)
+    assert f(5 * MB, 16, 64) == 5 * MB and f(w1, 4096, 64) == w1
