@@ -66,6 +66,10 @@ int32_t moeca_probe_hold(int32_t device, int32_t blocks, int32_t smem_bytes, int
  * moeca_config.weight_prefetch_mb = setting_mb.  Runs on the host. */
 int64_t moeca_probe_prefetch_bytes(int64_t w1_bytes, int32_t setting_mb, int32_t blocks);
 
+/* Tensor maps (TMA descriptors) this process has encoded, on any thread: host
+ * work, done once per handle for its own buffers. */
+int64_t moeca_probe_maps_encoded(void);
+
 #ifdef __cplusplus
 }
 #endif

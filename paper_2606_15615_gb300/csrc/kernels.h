@@ -260,11 +260,10 @@ cudaError_t launch_combine(const CombineArgs& a, bool bf16, cudaStream_t s);
 // Tensor-core projection GEMM: C = A B^T + bias (proj_tc.cu).
 enum ProjMode { kProjResidual = 1, kProjQKV = 2, kProjResidualGated = 3 };
 struct ProjArgs {
-  const void* A;          // [a_rows, K] bf16, row-major
+  const void* A;          // [a_rows, K] bf16, row-major, or null: the rows the plan was made for
   int a_rows;             // rows A holds (>= M)
-  const void* B;          // [N, K] bf16 weights
   const float* bias;      // [N] or null
-  int M, N, K;            // N a multiple of 64, K of 64
+  int M;
   const int* m_dev;       // device row count (<= M), or null
   int mode;               // ProjMode
   const int32_t* rows;    // kProjResidual: token of row m, or null (m)
@@ -286,7 +285,13 @@ struct ProjArgs {
                           //   written the weights, so that none load before the dependency wait
   int* status;
 };
-cudaError_t launch_proj_tc(const ProjArgs& a, int n_sms, cudaStream_t s);
+// The tensor maps of one weight matrix [N, K] (bf16; N and K multiples of 64)
+// and, unless A is null, of the rows A [a_rows, K] it is applied to: built once
+// per handle and layer.  Null on failure.
+struct ProjPlan;
+ProjPlan* proj_plan_create(const void* w, int N, int K, const void* A, int a_rows);
+void proj_plan_destroy(ProjPlan* p);
+cudaError_t launch_proj_tc(const ProjPlan* plan, const ProjArgs& a, int n_sms, cudaStream_t s);
 
 // ---- AdaLN modulation of a DiT-MoE block (Sec. 3) and the sampler step (Eq. 1) ----
 

@@ -91,6 +91,8 @@ struct LayerBuf {
   void* route_m = nullptr;   // [T, D] AdaLN block: its router input (keep_route_in)
   float* cache_y = nullptr;  // [T, D] fp32 each token's last computed MoE output (token_reuse_policy 1)
   TcPlan* tc = nullptr;
+  ProjPlan* qkv = nullptr;   // attention projections of a DiT-MoE block
+  ProjPlan* oproj = nullptr;
   bool valid = false;
 };
 
@@ -204,8 +206,11 @@ bool dev_alloc(moeca_handle* h, void** p, size_t bytes) {
 }
 
 void free_all(moeca_handle* h) {
-  for (auto& L : h->layers)
+  for (auto& L : h->layers) {
     if (L.tc) tc_plan_destroy(L.tc);
+    proj_plan_destroy(L.qkv);
+    proj_plan_destroy(L.oproj);
+  }
   auto& io = h->hio;
   for (int b = 0; b < 2; ++b) {
     if (io.up[b]) cudaEventDestroy(io.up[b]);
@@ -634,6 +639,17 @@ moeca_status moeca_create(const moeca_config* cfg, const moeca_layer_weights* la
       }
     }
   }
+  for (int l = 0; attn && l < c.n_layers; ++l) {
+    // The first block's input is each step's own, unless AdaLN forms it.
+    LayerBuf& L = h->layers[l];
+    L.qkv = proj_plan_create(L.w.w_qkv, 3 * c.hidden, c.hidden, ada ? h->ada_h : h->act[l], c.max_tokens);
+    L.oproj = proj_plan_create(L.w.w_o, c.hidden, c.hidden, h->attn_o, c.max_tokens);
+    if (!L.qkv || !L.oproj) {
+      free_all(h);
+      delete h;
+      return fail(nullptr, MOECA_ERR_CUDA, "projection plan: tensor map encoding failed");
+    }
+  }
   if ((ce = cudaDeviceSynchronize()) != cudaSuccess) {
     free_all(h);
     delete h;
@@ -718,15 +734,14 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
     void* k_buf = static_cast<char*>(h->qkv) + TD * h->es;
     void* vt_buf = static_cast<char*>(h->qkv) + 2 * TD * h->es;
     ProjArgs qa{};
-    qa.A = ada ? h->ada_h : in; qa.a_rows = T; qa.B = L.w.w_qkv; qa.bias = L.w.b_qkv;
-    qa.M = T; qa.N = 3 * c.hidden; qa.K = c.hidden; qa.mode = kProjQKV;
+    qa.A = l == 0 && !ada ? in : nullptr; qa.a_rows = T; qa.bias = L.w.b_qkv;
+    qa.M = T; qa.mode = kProjQKV;
     qa.q_out = q_buf; qa.k_out = k_buf; qa.vt_out = vt_buf; qa.n_tok = T; qa.status = h->status_dev;
     AttnArgs aa{};
     aa.q = q_buf; aa.k = k_buf; aa.vt = vt_buf; aa.T = T; aa.D = c.hidden; aa.H = c.n_heads; aa.S = seq;
     aa.o = h->attn_o; aa.status = h->status_dev;
     ProjArgs oa{};
-    oa.A = h->attn_o; oa.a_rows = T; oa.B = L.w.w_o; oa.bias = L.w.b_o;
-    oa.M = T; oa.N = c.hidden; oa.K = c.hidden; oa.mode = kProjResidual;
+    oa.bias = L.w.b_o; oa.M = T; oa.mode = kProjResidual;
     oa.n_tok = T; oa.x = in; oa.a_out = L.attn_a; oa.u_out = L.attn_u;
     if (ada) {
       oa.mode = kProjResidualGated;
@@ -746,11 +761,11 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
         ha.h_out = h->ada_h;
         if ((e = timed(h, MOECA_K_ADALN, s, [&] { return launch_adaln_rows(ha, s); })) != cudaSuccess) break;
       }
-      if ((e = timed(h, MOECA_K_QKV, s, [&] { return launch_proj_tc(qa, h->n_sms, s); })) != cudaSuccess) break;
+      if ((e = timed(h, MOECA_K_QKV, s, [&] { return launch_proj_tc(L.qkv, qa, h->n_sms, s); })) != cudaSuccess) break;
       if ((e = timed(h, MOECA_K_ATTN, s, [&] {
              return use_attn_tc ? launch_attn_tc(aa, s) : launch_attn_core(aa, s);
            })) != cudaSuccess) break;
-      if ((e = timed(h, MOECA_K_OPROJ, s, [&] { return launch_proj_tc(oa, h->n_sms, s); })) != cudaSuccess) break;
+      if ((e = timed(h, MOECA_K_OPROJ, s, [&] { return launch_proj_tc(L.oproj, oa, h->n_sms, s); })) != cudaSuccess) break;
       if (ada) {
         AdaLnArgs mm = la;
         mm.m_out = L.attn_m; mm.m_copy = L.route_m;
@@ -850,11 +865,11 @@ moeca_status moeca_step(moeca_handle* h, const void* x_in, void* x_out, const mo
                                                h->attn_inv, s);
                      })) != cudaSuccess)
         break;
-      if ((e = timed(h, MOECA_K_QKV, s, [&] { return launch_proj_tc(qa, h->n_sms, s); })) != cudaSuccess) break;
+      if ((e = timed(h, MOECA_K_QKV, s, [&] { return launch_proj_tc(L.qkv, qa, h->n_sms, s); })) != cudaSuccess) break;
       if ((e = timed(h, MOECA_K_ATTN, s, [&] {
              return use_attn_tc ? launch_attn_tc(aa, s) : launch_attn_core(aa, s);
            })) != cudaSuccess) break;
-      if ((e = timed(h, MOECA_K_OPROJ, s, [&] { return launch_proj_tc(oa, h->n_sms, s); })) != cudaSuccess) break;
+      if ((e = timed(h, MOECA_K_OPROJ, s, [&] { return launch_proj_tc(L.oproj, oa, h->n_sms, s); })) != cudaSuccess) break;
       if (ada) {
         // The listed tokens' MoE input m from their new u.
         AdaLnArgs mm = la;

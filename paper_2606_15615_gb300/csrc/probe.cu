@@ -7,8 +7,10 @@
 #include <algorithm>
 #include <vector>
 
+#include "common.cuh"
 #include "kernels.h"
 #include "moeca_probe.h"
+#include "tc_common.cuh"
 
 namespace {
 
@@ -225,3 +227,5 @@ extern "C" int64_t moeca_probe_prefetch_bytes(int64_t w1_bytes, int32_t setting_
   if (w1_bytes < 0 || setting_mb < 0 || blocks < 0) return -1;
   return static_cast<int64_t>(moeca::prep_prefetch_bytes(static_cast<size_t>(w1_bytes), setting_mb, blocks));
 }
+
+extern "C" int64_t moeca_probe_maps_encoded(void) { return moeca::g_maps_encoded.load(std::memory_order_relaxed); }

@@ -45,6 +45,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <new>
 #include <type_traits>
 
 #include "common.cuh"
@@ -103,7 +104,7 @@ struct ProjMaps {
 // Token tile width for `rows` rows: the fewest waves x time per tile.  A
 // tile's time per stage is its MMAs' (an M 256 MMA takes as long at N 128 as at
 // 256) plus a share that grows with the token rows brought in.
-__device__ __forceinline__ int token_width(int rows, int nw, int pairs) {
+__host__ __device__ __forceinline__ int token_width(int rows, int nw, int pairs) {
   int best = 256, best_cost = 0x7fffffff;
   for (int n = 256; n >= 32; n -= 32) {
     const int tiles = (rows + n - 1) / n * nw;
@@ -477,17 +478,52 @@ __global__ void __launch_bounds__(kPThreads, 1)
 
 }  // namespace
 
-cudaError_t launch_proj_tc(const ProjArgs& a, int n_sms, cudaStream_t s) {
-  if (a.N % 64 || a.K % 64 || a.M <= 0) return cudaErrorInvalidValue;
-  if (a.mode == kProjResidualGated && (!a.gate || a.seq <= 0 || a.row_of)) return cudaErrorInvalidValue;
+struct ProjPlan {
   ProjMaps maps;
-  if (!encode_k64(&maps.w, a.B, static_cast<uint64_t>(a.N), static_cast<uint64_t>(a.K), kBM, kSub))
-    return cudaErrorInvalidValue;
-  for (int i = 0; i < kBoxes; ++i)
-    if (!encode_k64(&maps.act[i], a.A, static_cast<uint64_t>(a.a_rows), static_cast<uint64_t>(a.K), 16 * (i + 1), kSub))
-      return cudaErrorInvalidValue;
+  int N, K;
+  bool rows;  // the token maps are set
+};
+
+ProjPlan* proj_plan_create(const void* w, int N, int K, const void* A, int a_rows) {
+  if (N % 64 || K % 64) return nullptr;
+  ProjPlan* p = new (std::nothrow) ProjPlan{};
+  if (!p) return nullptr;
+  p->N = N;
+  p->K = K;
+  p->rows = A != nullptr;
+  bool ok = encode_k64(&p->maps.w, w, static_cast<uint64_t>(N), static_cast<uint64_t>(K), kBM, kSub);
+  for (int i = 0; i < kBoxes && ok && A; ++i)
+    ok = encode_k64(&p->maps.act[i], A, static_cast<uint64_t>(a_rows), static_cast<uint64_t>(K), 16 * (i + 1), kSub);
+  if (ok) return p;
+  delete p;
+  return nullptr;
+}
+
+void proj_plan_destroy(ProjPlan* p) { delete p; }
+
+cudaError_t launch_proj_tc(const ProjPlan* plan, const ProjArgs& a, int n_sms, cudaStream_t s) {
+  if (!plan || a.M <= 0 || (!a.A && !plan->rows)) return cudaErrorInvalidValue;
+  if (a.mode == kProjResidualGated && (!a.gate || a.seq <= 0 || a.row_of)) return cudaErrorInvalidValue;
+  const int N = plan->N, K = plan->K;
+  // At most one pair per tile of the narrowest width.
+  const int nw = (N + 2 * kBM - 1) / (2 * kBM);
+  const int pairs = std::max(1, std::min(n_sms / 2, (a.M + 31) / 32 * nw));
+  ProjMaps maps = plan->maps;
+  if (a.A) {
+    // The caller's rows (a step's input): the one width the launch will take
+    // when the host knows the row count, else all of them.
+    const int only = a.m_dev ? 0 : token_width(a.M, nw, pairs) / 32;
+    for (int i = 0; i < kBoxes; ++i) {
+      if (only && i) {
+        maps.act[i] = maps.act[0];
+      } else if (!encode_k64(&maps.act[i], a.A, static_cast<uint64_t>(a.a_rows), static_cast<uint64_t>(K),
+                             16 * (only ? only : i + 1), kSub)) {
+        return cudaErrorInvalidValue;
+      }
+    }
+  }
   ProjParams p{};
-  p.M = a.M; p.N = a.N; p.K = a.K; p.m_dev = a.m_dev; p.bias = a.bias;
+  p.M = a.M; p.N = N; p.K = K; p.m_dev = a.m_dev; p.bias = a.bias;
   p.rows = a.rows; p.n_tok = a.n_tok;
   p.x = static_cast<const __nv_bfloat16*>(a.x);
   p.a_out = static_cast<__nv_bfloat16*>(a.a_out);
@@ -503,9 +539,6 @@ cudaError_t launch_proj_tc(const ProjArgs& a, int n_sms, cudaStream_t s) {
   p.gate = a.gate; p.gate_ld = a.gate_ld; p.seq = a.seq;
   p.first = a.first;
   p.status = a.status;
-  // At most one pair per tile of the narrowest width.
-  const int nw = (a.N + 2 * kBM - 1) / (2 * kBM);
-  const int pairs = std::max(1, std::min(n_sms / 2, (a.M + 31) / 32 * nw));
   auto run = [&](auto kern) -> cudaError_t {
     const cudaError_t e = set_dyn_smem_on_device(reinterpret_cast<const void*>(kern), kPSmem);
     if (e != cudaSuccess) return e;

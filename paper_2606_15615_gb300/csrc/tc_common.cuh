@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace moeca {
 
 // Every bounded wait of the tensor-core kernels gives up after this long.
@@ -215,6 +217,9 @@ inline EncodeTiledFn get_encoder() {
   return fn;
 }
 
+// Maps encoded by this process (host work a step should not repeat for its own buffers).
+inline std::atomic<long long> g_maps_encoded{0};
+
 // 2-D bf16 map over [rows, cols] row-major, box {64, box_rows}, 128-byte swizzle.
 inline bool encode_2d(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
   EncodeTiledFn enc = get_encoder();
@@ -223,6 +228,7 @@ inline bool encode_2d(CUtensorMap* m, const void* base, uint64_t rows, uint64_t 
   cuuint64_t strides[1] = {cols * 2};
   cuuint32_t box[2] = {static_cast<cuuint32_t>(64), box_rows};
   cuuint32_t estr[2] = {1, 1};
+  g_maps_encoded.fetch_add(1, std::memory_order_relaxed);
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -240,6 +246,7 @@ inline bool encode_k64(CUtensorMap* m, const void* base, uint64_t rows, uint64_t
   cuuint64_t strides[2] = {cols * 2, 128};
   cuuint32_t box[3] = {64, box_rows, subs};
   cuuint32_t estr[3] = {1, 1, 1};
+  g_maps_encoded.fetch_add(1, std::memory_order_relaxed);
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;

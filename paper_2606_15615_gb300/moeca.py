@@ -144,6 +144,7 @@ def _load():
                                           C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_double)]),
         "moeca_ddpm_step": (C.c_int, [C.POINTER(moeca_ddpm_args), C.c_void_p]),
         "moeca_probe_ffma": (C.c_int32, [C.c_int32, C.c_int32, C.POINTER(C.c_double), C.POINTER(C.c_double)]),
+        "moeca_probe_maps_encoded": (C.c_int64, []),
         "moeca_probe_prefetch_bytes": (C.c_int64, [C.c_int64, C.c_int32, C.c_int32]),
         "moeca_probe_hold": (C.c_int32, [C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_void_p]),
         "moeca_probe_stream": (C.c_int32, [C.c_int32, C.c_int64, C.c_int32, C.c_int32, C.c_int32,

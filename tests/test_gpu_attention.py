@@ -278,3 +278,28 @@ def test_full_step_sees_projection_weights_a_kernel_just_before_wrote(M):
         st.close()
     for a, b in zip(outs[:6], outs[6:]):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("L", [1, 3])
+def test_projection_maps_are_built_once(M, L):
+    """Steps of a block stack encode one tensor map each, of the step's input
+    (the warp-level attention core has none), not several per layer: the other
+    projections read the handle's buffers.  Inputs in changing buffers and
+    token counts below max_tokens, with the results of a handle of that size."""
+    D, H, S = 256, 4, 40
+    rng = np.random.default_rng(170)
+    big, _, _ = make_block_stack(M, 240, D, H, 8, 2, 256, L=L, S=S, seed=17, tau0=0.72, attn_impl=1)
+    for T in (120, 200, 40):
+        ref, _, _ = make_block_stack(M, T, D, H, 8, 2, 256, L=L, S=S, seed=17, tau0=0.72, attn_impl=1)
+        xs = [torch.from_numpy(x).cuda().to(torch.bfloat16)
+              for x in drift(rng.standard_normal((T, D)).astype(np.float32), rng, 3, 0.1)]
+        want = [ref.step(x, t) for t, x in enumerate(xs)]
+        before = M.LIB.moeca_probe_maps_encoded()
+        got = [big.step(x, t) for t, x in enumerate(xs)]
+        assert M.LIB.moeca_probe_maps_encoded() - before == len(xs)
+        torch.cuda.synchronize()
+        assert ref.stats()["attn_recomputed"] > 0
+        for a, b in zip(want, got):
+            assert torch.equal(a, b)
+        ref.close()
+    big.close()
