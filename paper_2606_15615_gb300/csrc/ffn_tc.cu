@@ -76,7 +76,7 @@ constexpr int kBM = 128;          // weight rows per CTA (half of the MMA's M)
 constexpr int kBK = 64;           // K per sub-block: 64 bf16 = one 128-byte swizzle row
 constexpr int kSub = 2;           // K sub-blocks per stage
 constexpr int kMaxN = 256;        // token rows per tile
-constexpr int kMaxStages = 11;
+constexpr int kMaxStages = 5;     // what the ring holds at the narrowest token tile (32 rows)
 constexpr int kRingBytes = 208 * 1024;  // beside 16 KB of epilogue stages
 constexpr int kEpiWarps = 8;        // warps 2-9
 constexpr int kTokWarp = 2 + kEpiWarps;
@@ -86,6 +86,7 @@ constexpr int kTmemCols = 512;
 constexpr int kABytes = kBM * kBK * 2;  // 16 KB: one weight sub-block
 constexpr int kStageOut = 32 * 64;      // per epilogue warp: 32 tokens x 32 features of bf16
 constexpr int kSmemBytes = kRingBytes + kEpiWarps * kStageOut + 1024;
+static_assert(kMaxStages == kRingBytes / (kSub * (kABytes + 32 / 2 * (kBK * 2))), "stages at the narrowest tile");
 constexpr int kMaxGroups = kMaxExperts + 1;
 constexpr unsigned long long kWaitNs = 1000000000ull;
 constexpr int kUQ = 4;            // unit queue from the leader's producer to the other roles
@@ -131,27 +132,6 @@ __device__ __forceinline__ float gelu_tanh_hw(float z) {
   asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(u));
   const float hz = 0.5f * z;
   return fmaf(hz, t, hz);
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t*>(&h2);
-}
-
-// A warp's 32 features x 32 tokens of the accumulator (lane = feature), as
-// bf16 into the stage [32 tokens][32 features].  Lanes 2i and 2i + 1 swap
-// halves, so that each holds the feature pair of every other token: the even
-// lane tokens 0, 2, .., the odd lane 1, 3, ..; the 32 words of each store
-// then fall in 32 banks.
-__device__ __forceinline__ void stage_chunk(uint32_t* stage, const uint32_t* v, int lane) {
-  const uint32_t odd = lane & 1;
-#pragma unroll
-  for (int t = 0; t < 16; ++t) {
-    const uint32_t own = pack_bf16(__uint_as_float(v[2 * t]), __uint_as_float(v[2 * t + 1]));
-    const uint32_t got = __shfl_xor_sync(0xffffffffu, own, 1);
-    const uint32_t word = odd ? __byte_perm(got, own, 0x7632) : __byte_perm(own, got, 0x5410);
-    stage[(2 * t + odd) * 16 + (lane >> 1)] = word;
-  }
 }
 
 // A phase's geometry for this launch.
@@ -265,7 +245,7 @@ __device__ __forceinline__ void store32(uint32_t* v, int c, int c_lo, int c_hi, 
     }
   }
   __syncwarp();
-  stage_chunk(stage, v, lane);
+  stage_by_token(stage, lane, [&](int t) { return __uint_as_float(v[t]); });
   __syncwarp();
   const int src = (c - c_lo) >> 5;
   const int d = src == 0 ? dr.x : (src == 1 ? dr.y : (src == 2 ? dr.z : dr.w));
@@ -279,8 +259,9 @@ __device__ __forceinline__ void store32(uint32_t* v, int c, int c_lo, int c_hi, 
   }
 }
 
-// A warp's part of a finished tile, columns [c_lo, c_hi), from TMEM to memory;
-// the next chunk's TMEM load is in flight while this one is stored.
+// A warp's part of a finished tile, columns [c_lo, c_hi), from TMEM to memory,
+// 32 columns at a time (each chunk's load is waited for: the eight warps of a
+// CTA hide it for each other).
 template <bool TANH>
 __device__ __forceinline__ void store_tile(uint32_t tb, int c_lo, int c_hi, int p, int row0, int4 dr, __nv_bfloat16* base,
                                         int N, uint32_t* stage) {

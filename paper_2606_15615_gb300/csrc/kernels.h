@@ -90,7 +90,7 @@ struct CompactArgs {
   const int32_t* offsets;
   int32_t* list;        // [rows]
   const void* x;        // [T, D]
-  void* xg;             // [rows, D] gathered inputs, or null when the GEMM gathers itself
+  void* xg;             // [rows, D] gathered inputs, or null: gathered later (launch_gather)
   int* status;
 };
 // compact_kernel (row lists), then, unless xg is null, gather_kernel (rows).
@@ -138,7 +138,7 @@ struct FfnArgs {
   void* shared_h;        // [T, D]     destination rows of the shared group
   int gelu_tanh;
   int tile_n;            // tensor-core path: widest token tile to force (0: 256)
-  int split_k;           // tensor-core K splits to force (0: chosen per launch)
+  int split_k;           // tensor-core path: K splits of the second GEMM to force (0: none)
   float* partial;        // split-K workspace: tensor-core path, or the fp32 path's [simt_split, max_rows, D]
   int simt_split;        // fp32 path: K splits of the second GEMM (1: none)
   int* tile_sem;         // split-K arrival counters, zeroed once
@@ -161,7 +161,8 @@ void tc_plan_destroy(TcPlan* p);
 // Both GEMMs in one persistent launch.
 cudaError_t launch_ffn_tc(TcPlan* p, const FfnArgs& a, cudaStream_t s);
 
-// Fused router + select + compact (one cooperative launch, bf16 only).
+// Fused router + select + compact (bf16 only): one launch whose blocks are all
+// resident and exchange values, under the programmatic dependency.
 struct PrepArgs {
   const void* x;          // [T, D] layer input
   const void* w_gate;     // [E, D]

@@ -102,8 +102,10 @@ struct ProjMaps {
 };
 
 // Token tile width for `rows` rows: the fewest waves x time per tile.  A
-// tile's time per stage is its MMAs' (an M 256 MMA takes as long at N 128 as at
-// 256) plus a share that grows with the token rows brought in.
+// tile's time per stage is modelled as 384 + n: the MMAs alone take n / 2
+// clocks each (64 at 128 columns, 128 at 256, at least 45), but the
+// single-thread roles' work per stage and the barrier round trips do not
+// depend on n, so that narrow tiles save less than their share.
 __host__ __device__ __forceinline__ int token_width(int rows, int nw, int pairs) {
   int best = 256, best_cost = 0x7fffffff;
   for (int n = 256; n >= 32; n -= 32) {
@@ -117,26 +119,8 @@ __host__ __device__ __forceinline__ int token_width(int rows, int nw, int pairs)
   return best;
 }
 
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t*>(&h2);
-}
-
-// A warp's 32 features (lanes) x 32 tokens as bf16 into the stage
-// [32 tokens][32 features]: lanes 2i and 2i + 1 swap halves, so that each holds
-// the feature pair of every other token and the 32 words of a store fall in
-// 32 banks.
-__device__ __forceinline__ void stage_by_token(uint32_t* stage, const uint32_t* v, float bias, int lane) {
-  const uint32_t odd = lane & 1;
-#pragma unroll
-  for (int t = 0; t < 16; ++t) {
-    const uint32_t own = pack_bf16(__uint_as_float(v[2 * t]) + bias, __uint_as_float(v[2 * t + 1]) + bias);
-    const uint32_t got = __shfl_xor_sync(0xffffffffu, own, 1);
-    stage[(2 * t + odd) * 16 + (lane >> 1)] = odd ? __byte_perm(got, own, 0x7632) : __byte_perm(own, got, 0x5410);
-  }
-}
-
-// The same as [32 features][32 tokens], 16-byte chunks XOR-swizzled by row
+// A warp's 32 features (lanes) x 32 tokens as bf16 into the stage as
+// [32 features][32 tokens], 16-byte chunks XOR-swizzled by row
 // pairs so that both accesses are conflict-free.
 __device__ __forceinline__ void stage_by_feature(uint32_t* stage, const uint32_t* v, float bias, int lane) {
 #pragma unroll
@@ -383,7 +367,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
           }
           tmem_wait32(v);
           __syncwarp();
-          stage_by_token(stage, v, bias, lane);
+          stage_by_token(stage, lane, [&](int t) { return __uint_as_float(v[t]) + bias; });
           __syncwarp();
 #pragma unroll
           for (int it = 0; it < 4; ++it) {
@@ -427,7 +411,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
           tmem_wait32(v);
           __syncwarp();
           if (region < 2) {
-            stage_by_token(stage, v, bias, lane);
+            stage_by_token(stage, lane, [&](int t) { return __uint_as_float(v[t]) + bias; });
             __syncwarp();
             __nv_bfloat16* base = (region == 0 ? p.q_out : p.k_out) + f + s_ch * 8;
 #pragma unroll

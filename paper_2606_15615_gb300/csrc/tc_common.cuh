@@ -5,6 +5,7 @@
 #pragma once
 
 #include <cuda.h>
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -198,6 +199,27 @@ __device__ __forceinline__ void tmem_wait32(uint32_t* v) {
                  "+r"(v[30]), "+r"(v[31])
                :
                : "memory");
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<uint32_t*>(&h2);
+}
+
+// A warp's 32 features (lanes) x 32 tokens (value(t), t < 32) as bf16 into the
+// stage [32 tokens][32 features].  Lanes 2i and 2i + 1 swap halves, so that each
+// holds the feature pair of every other token: the even lane tokens 0, 2, ..,
+// the odd lane 1, 3, ..; the 32 words of each store then fall in 32 banks.
+template <typename F>
+__device__ __forceinline__ void stage_by_token(uint32_t* stage, int lane, F value) {
+  const uint32_t odd = lane & 1;
+#pragma unroll
+  for (int t = 0; t < 16; ++t) {
+    const uint32_t own = pack_bf16(value(2 * t), value(2 * t + 1));
+    const uint32_t got = __shfl_xor_sync(0xffffffffu, own, 1);
+    const uint32_t word = odd ? __byte_perm(got, own, 0x7632) : __byte_perm(own, got, 0x5410);
+    stage[(2 * t + odd) * 16 + (lane >> 1)] = word;
+  }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
