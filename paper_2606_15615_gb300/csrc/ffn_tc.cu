@@ -291,8 +291,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ uint32_t tmem_base_sh;
   __shared__ Groups gr;
   __shared__ int nmax_sh;
-  __shared__ __align__(8) uint64_t ticket_bar;  // the peer's: the pair's first ticket is there
-  __shared__ int ticket_sh;
+  __shared__ int ticket_sh;  // leader's: the pair's first ticket
   __shared__ volatile int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -312,8 +311,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(smem_u32(&tempty_bar[s]), 2 * kEpiWarps);
     }
     mbar_init(smem_u32(&drain_bar), 1);
-    mbar_init(smem_u32(&ticket_bar), 1);
-    mbar_expect_tx(smem_u32(&ticket_bar), 4);
     for (int q = 0; q < kUQ; ++q) {
       mbar_init(smem_u32(&uq_full[q]), 1);
       mbar_init(smem_u32(&pub_bar[q]), kEpiWarps);
@@ -329,6 +326,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                  ::"r"(smem_u32(&tmem_base_sh)), "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     tc_fence_before();
+    // The pair's first ticket.  The counter was re-armed by a combine that lies
+    // before the previous kernel, which has passed its own wait.
+    if (lane == 0 && rank == 0) ticket_sh = atomicAdd(a.work, 1);
   }
   if (warp == 2 && lane < 2 * (kBoxes + 2)) {
     const TcMaps& m = maps.p[lane & 1];
@@ -343,26 +343,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                  "l"(a.counts), "l"(a.offsets), "l"(a.list), "l"(a.hmid), "l"(a.dep), "l"(a.cache_h), "l"(a.work),
                  "r"(a.E), "r"(a.dep_pairs));
   }
-  // The pair's first ticket.  The counter was re-armed by a combine that lies
-  // before the previous kernel, which has passed its own wait.  Drawn this
-  // early by a warp that has nothing to release, the ticket costs at most 0.5 us
-  // a launch against first units fixed to the pair's index (D 768, 2048 tokens,
-  // 4 layer steps 278.7 -> 280.7 us; 0.9 us with the draw in warp 0, and as much
-  // with fixed first units that other pairs can take: code that runs first
-  // after the wait is fetched while the weights stream in).
-  int drawn = 0;
-  if (warp == 3) {
-    if (lane == 0 && rank == 0) drawn = atomicAdd(a.work, 1);
-    cluster_arrive_relaxed();
-  } else {
-    cluster_arrive();
-  }
-  cluster_wait();  // both CTAs' barriers are initialised
-  if (warp == 3 && lane == 0 && rank == 0) {
-    // To both CTAs' weight producers.
-    st_async_cluster(cluster_addr(smem_u32(&ticket_sh), 1), drawn, cluster_addr(smem_u32(&ticket_bar), 1));
-    ticket_sh = drawn;
-  }
+  cluster_arrive();
+  cluster_wait();  // both CTAs' barriers are initialised, the leader has its ticket
+  // The weight producers' next unit (after the first, the leader's alone).  The
+  // draw and its way to the peer lie before the dependency wait (code that runs
+  // first after it is fetched while the weights stream in: an mbarrier or the
+  // unit queue there cost 1.2 us a launch), and the draw follows the TMEM
+  // allocation (drawn by other warps it cost 0.5 to 2 us).  So placed it costs
+  // nothing against first units fixed to the pair's index (12-layer D 768 stack
+  // 0.747 -> 0.748 ms a step; one layer of it, four steps, 279 -> 278 us).
+  int ticket = 0;
+  if (threadIdx.x == 0) ticket = ld_cluster(cluster_addr(smem_u32(&ticket_sh), 0));
   Phase p0, p1;
   p0.nw = (a.N[0] + 255) >> 8;
   p1.nw = (a.N[1] + 255) >> 8;
@@ -459,10 +450,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         return true;
       };
-      // The first unit does without the queue: the peer decodes its ticket too.
-      if (!leader)
-        ok = mbar_try_cluster(smem_u32(&ticket_bar), 0) || mbar_wait_cluster(smem_u32(&ticket_bar), 0, &abort_flag);
-      int ticket = *static_cast<volatile int*>(&ticket_sh);
+      // The first unit does without the queue: both CTAs have its ticket.
       int4 cur = unit_word(ticket, total, p0, p1, gr, G);
       if (leader) ok = push(cur);
       for (bool first = true; ok; first = false) {

@@ -108,8 +108,6 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
   return r;
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-// As cluster_arrive for a warp with nothing to release: does not wait for its memory operations in flight.
-__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // Arrive on a barrier of either CTA (a shared::cluster address), releasing this thread's writes to the cluster.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
@@ -119,26 +117,23 @@ __device__ __forceinline__ void st_cluster(uint32_t addr, const int4& v) {
   asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
                : "memory");
 }
-// A word into a CTA's shared memory (shared::cluster addresses), its 4 bytes completing on that CTA's barrier.
-__device__ __forceinline__ void st_async_cluster(uint32_t addr, int v, uint32_t bar) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar)
-               : "memory");
+__device__ __forceinline__ int ld_cluster(uint32_t addr) {
+  int v;
+  asm volatile("ld.shared::cluster.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
 }
-// As mbar_try and mbar_wait, acquiring what a thread of the other CTA released.
-__device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
+// As mbar_wait, acquiring what a thread of the other CTA released.
 static __device__ __noinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   unsigned long long t0 = 0;
   for (uint32_t it = 1;; ++it) {
-    if (mbar_try_cluster(bar, parity)) return true;
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
     if ((it & 255u) == 0) {
       if (*abort_flag) return false;
       const unsigned long long now = globaltimer();
