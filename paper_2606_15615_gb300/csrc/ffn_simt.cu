@@ -326,10 +326,11 @@ __global__ void __launch_bounds__(256) ffn_split_sum_kernel(FfnArgs a) {
 // once, each striding over the launch's tiles, so that they can be launched
 // early under the programmatic dependency: a grid of the worst case's blocks
 // sat beside the previous kernel's and slowed them (fp32 workload: 455 vs
-// 209 us per step), and plain launches left the gaps between the kernels open
-// (4 steps, D 384, 512 tokens, side by side: 380 -> 366 us with the decision
-// kernel's part in it).  The plain form keeps the worst case's grid and plain
-// launches.
+// 209 us per step).  Against plain launches of the worst case's grids, measured
+// side by side: steps back to back 95.6 -> 92.4 us (D 384, 8 experts, 512
+// tokens), small steps 173 -> 164 us a pass (61 tokens), but a pass of 4 steps
+// at 512 tokens with other kernels between them 344 -> 357 us.  The plain form
+// keeps the worst case's grid and plain launches.
 template <typename TI>
 cudaError_t launch_t(const FfnArgs& a, int phase, int n_sms, cudaStream_t s) {
   const int N = phase == 1 ? a.F : a.D;
