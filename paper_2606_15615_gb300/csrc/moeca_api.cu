@@ -124,7 +124,7 @@ struct moeca_handle {
   int simt_split = 1;
   int* tc_sem = nullptr;
   int* tc_dep = nullptr;        // grouped GEMM: token-tile dependency counters, left at 0
-  int* tc_work = nullptr;       // GEMM unit tickets {next, CTAs done}, left at 0
+  int* tc_work = nullptr;       // grouped GEMM: unit ticket counter, left at 0
   int tc_dep_pairs_n = 0;
   PrepShape prep{0, 0, 0, 0, false};  // fused router + select + compact, when it fits
   int decide_blocks = 0;        // separate path: decide_kernel's blocks at max_tokens (0: the three kernels)
@@ -588,7 +588,7 @@ moeca_status moeca_create(const moeca_config* cfg, const moeca_layer_weights* la
     A((void**)&h->tc_sem, tc_split_sems(h->n_sms) * sizeof(int));
     h->tc_dep_pairs_n = static_cast<int>(tc_dep_pairs(h->max_rows, h->G));
     A((void**)&h->tc_dep, static_cast<size_t>(h->tc_dep_pairs_n) * 2 * sizeof(int));
-    A((void**)&h->tc_work, 2 * sizeof(int));
+    A((void**)&h->tc_work, sizeof(int));
     // An AdaLN block forms its router input in its own kernel.
     h->prep = prep_plan(c.hidden, c.n_experts, c.top_k, c.max_tokens, h->n_sms, attn, attn && !ada);
     if (h->prep.tokens_per_block) {
@@ -1277,7 +1277,7 @@ moeca_status moeca_reset(moeca_handle* h) {
   if (h->tc_dep) {
     cudaError_t e = cudaMemset(h->tc_dep, 0, static_cast<size_t>(h->tc_dep_pairs_n) * 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->tc_sem, 0, tc_split_sems(h->n_sms) * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(h->tc_work, 0, 2 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(h->tc_work, 0, sizeof(int));
     if (e != cudaSuccess) return cuda_fail(h, e, "reset GEMM counters");
   }
   for (auto& L : h->layers) {

@@ -498,6 +498,37 @@ def test_ffn_pairs_kept_off_the_gpu_hold_up_nobody(M, E, F):
         assert torch.equal(o, outs[0])
 
 
+def test_two_handles_on_two_streams(M):
+    """A stack run by the preparation kernel and one run by the router and the
+    decision kernel, at sizes that fill the GPU, stepping at the same time on
+    two streams: both kernels wait for their own blocks, and the FFN's pairs
+    for each other's tiles.  The bits of handles that step alone, no status."""
+    shapes = [(2048, 768, 16, 2, 1024), (4096, 1152, 64, 8, 256)]
+    made = []
+    for n, (T, D, E, k, F) in enumerate(shapes):
+        w, x0, rng = W.tiny_layer(461 + n, T, D, E, k, F, dtype="bf16", wscale=0.02)
+        cfg = M.moeca_config_default(n_layers=1, hidden=D, ffn=F, n_experts=E, top_k=k, max_tokens=T,
+                                     dtype=M.MOECA_BF16, tau0=1.4 / k, refresh_period=8)
+        xs = [torch.from_numpy(x).cuda().to(torch.bfloat16) for x in drift(x0, rng, 8, 0.05, True)]
+        alone = M.Stack(cfg, [w])
+        want = [alone.step(xs[t % 8], t) for t in range(48)]
+        torch.cuda.synchronize()
+        assert 0 < alone.stats()["reused"] < alone.stats()["cache_step_branches"]
+        alone.close()
+        made.append((M.Stack(cfg, [w]), xs, want, torch.cuda.Stream(), []))
+    torch.cuda.synchronize()
+    for t in range(48):
+        for st, xs, _, stream, got in made:
+            with torch.cuda.stream(stream):
+                got.append(st.step(xs[t % 8], t))
+    torch.cuda.synchronize()
+    for st, _, want, _, got in made:
+        st.stats()  # raises if a wait ran out
+        st.close()
+        for a, b in zip(want, got):
+            assert torch.equal(a, b)
+
+
 def test_fp32_ffn_more_tiles_than_blocks(M):
     """2500 rows per expert: the fp32 FFN's blocks each take several tiles."""
     T, D, E, k, F = 5000, 64, 4, 2, 1024
