@@ -479,9 +479,9 @@ moeca_status moeca_destroy(moeca_handle* h);
  * at zero by the call before and set there anew by each call.  Calls that overlap
  * on the GPU (on different streams or from different host threads) race on the
  * scratch: serialise them.  Overlapping calls spoil their own outputs; the next
- * call after them is right again (a replayed capture, whose counter is only the
- * one left to it, after one such call).  Calls on one stream are ordered: each
- * sees what the one before, and any other work before it, wrote to its inputs.
+ * call launched directly (not replayed from a captured graph) is right again, and
+ * so are replays after it.  Calls on one stream are ordered: each sees what the
+ * one before, and any other work before it, wrote to its inputs.
  * Runs on the current device, asynchronously on `stream`. */
 typedef struct {
   int32_t dtype;         /* moeca_dtype of x and w_gate                       */
